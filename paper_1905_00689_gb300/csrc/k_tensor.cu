@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
   };
 
-  if (warp == 0 && lane == 0) {  // ---- TMA producer ----
+  if (warp == 0 && elect_one()) {  // ---- TMA producer ----
     tma_prefetch_map(&tma);
     tma_prefetch_map(&tmb);
     int issued = 0;
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const int last = s + ((issued - 1 - s) / S) * S;
       wait_cta(bar0 + 8u * s, (last / S) & 1, limit, err);
     }
-  } else if (warp == 1 && lane == 0) {  // ---- MMA issuer ----
+  } else if (warp == 1 && elect_one()) {  // ---- MMA issuer ----
     constexpr uint32_t idesc = umma_idesc_bf16(kTileM, BN);
     bool ok = true;
     for (int i = 0; i < nloc && ok; ++i) {
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {  // ---- TMA producer: stage i = (chunk i/4, gate i%4) ----
+  if (warp == 0 && elect_one()) {  // ---- TMA producer: stage i = (chunk i/4, gate i%4) ----
     tma_prefetch_map(&tmu);
     tma_prefetch_map(&tmt);
     const int nst = 4 * nkb;
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const int last = s + ((issued - 1 - s) / S) * S;
       wait_cta(bar0 + 8u * s, (last / S) & 1, limit, err);
     }
-  } else if (warp == 1 && lane == 0) {  // ---- MMA issuer ----
+  } else if (warp == 1 && elect_one()) {  // ---- MMA issuer ----
     constexpr uint32_t idesc = umma_idesc_bf16(kTileM, NT);
     bool ok = true;
     int jj = jj_lo;

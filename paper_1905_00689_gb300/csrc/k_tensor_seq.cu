@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(seq_threads(NS), 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {  // ---- factor copies, then the MMA issue of every step ----
+    if (elect_one()) {  // ---- factor copies, then the MMA issue of every step ----
       tma_prefetch_map(&tmv);
       tma_prefetch_map(&tmu);
       mbar_arrive_expect_tx(fac_full, (uint32_t)NU * R4 * 128u + 4u * MT * 8192u);
