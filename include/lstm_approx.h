@@ -265,8 +265,10 @@ enum lstm_approx_query_key {
   LSTM_APPROX_Q_DEVICE_BYTES = 3, /* device bytes currently held by the handle */
   LSTM_APPROX_Q_PERSISTENT_VARIANT = 4, /* persistent kernel of the last persistent run
                                           (1 or 2, see LSTM_APPROX_OPT_PERSISTENT_VARIANT) */
-  LSTM_APPROX_Q_TENSOR_SEQ = 5   /* 1 if the last tensor-path layer ran as one launch
-                                    for all timesteps (see LSTM_APPROX_OPT_TENSOR_SEQ) */
+  LSTM_APPROX_Q_TENSOR_SEQ = 5,  /* 1 if the last tensor-path layer ran as one launch per
+                                    stream tile for all timesteps (see LSTM_APPROX_OPT_TENSOR_SEQ) */
+  LSTM_APPROX_Q_TENSOR_LOOP = 6  /* 1 if it ran as one launch over all stream tiles for all
+                                    timesteps, its factors resident on chip */
 };
 enum lstm_approx_path {
   LSTM_APPROX_PATH_NONE = 0,
@@ -305,8 +307,10 @@ enum lstm_approx_option_key {
                                tile of streams for all T timesteps where the
                                layer fits: K <= 32, H = 256, 512 or 1024,
                                intermediate depths multiples of 16 or >= K,
-                               masked-dense tau'), 1 = two launches per
-                               timestep */
+                               masked-dense tau'; else one launch over all
+                               tiles for all T where the factors and the
+                               streams fit the GPU's CTAs: H <= 2048,
+                               K <= 1024), 1 = two launches per timestep */
   LSTM_APPROX_OPT_LAUNCH_ORDER = 9 /* batch-1 fp32 path with the per-unit-block
                                kernel: 0 = automatic (the recurrence is
                                launched before its input projection and
@@ -381,7 +385,11 @@ enum lstm_approx_plan_item {
                                               per timestep */
   LSTM_APPROX_PLAN_TAU_SPLITS = 14,        /* tensor path: CTAs of a cluster over which the tau'
                                               GEMM splits its reduction axis (H), 1 = none */
-  LSTM_APPROX_PLAN_ITEMS = 15
+  LSTM_APPROX_PLAN_TENSOR_LOOP = 15,       /* tensor path: 1 = one launch over all stream tiles for all
+                                              T (the tile and split items then describe the
+                                              per-timestep kernels that serve where the device cannot
+                                              hold that launch at once) */
+  LSTM_APPROX_PLAN_ITEMS = 16
 };
 int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int *checkpoints, int J,
                      int force_path, int cluster, int persistent_variant, int *out, int n_out,

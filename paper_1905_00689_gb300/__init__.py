@@ -12,5 +12,6 @@ from ._binding import (  # noqa: F401
     PATH_NONE, PATH_PERSISTENT, PATH_SIMT, PATH_TENSOR,
     OPT_CLUSTER, OPT_FORCE_PATH, OPT_LAUNCH_ORDER, OPT_PERSISTENT_VARIANT, OPT_TAU_LAYOUT, OPT_TENSOR_SEQ,
     OPT_TEST_STALL, OPT_TIMING, OPT_WAIT_LIMIT, OPT_XPROJ,
-    Q_CLUSTER, Q_DEVICE_BYTES, Q_LAST_PATH, Q_LAUNCHES, Q_PERSISTENT_VARIANT, Q_TENSOR_SEQ,
+    Q_CLUSTER, Q_DEVICE_BYTES, Q_LAST_PATH, Q_LAUNCHES, Q_PERSISTENT_VARIANT, Q_TENSOR_LOOP,
+    Q_TENSOR_SEQ,
 )

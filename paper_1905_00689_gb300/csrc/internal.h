@@ -93,6 +93,8 @@ struct lstm_approx {
   int* err_host = nullptr;    // pinned host copy of it, read after the stream synchronises
   unsigned* proj_flags = nullptr;  // [kProjFlags] completion flags of a projection launched after the recurrence
   unsigned proj_epoch = 0;         // the value the last such launch wrote
+  unsigned* loop_counts = nullptr;  // (after the flags) counters of the resident-factor tensor launch: h and tau' per
+                                    // stream tile, done
 
   // staging for lstm_approx_run_host
   size_t stage_bytes = 0;
@@ -110,7 +112,8 @@ struct lstm_approx {
   int opt_test_stall = 0;
   long long launches = 0;
   int last_path = 0, last_cluster = 0, last_variant = 0;
-  int last_tensor_seq = 0;  // 1 if the last tensor-path layer ran as one launch for all timesteps
+  int last_tensor_seq = 0;  // 1 if the last tensor-path layer ran as one launch per stream tile for all timesteps
+  int last_tensor_loop = 0;  // 1 if it ran as one launch over all stream tiles for all timesteps
   long long device_bytes = 0;
   lstm_approx_impl::Timing timing;
   std::string last_error;
@@ -378,6 +381,73 @@ bool tc_seq_fits(int H, int B, int K, const Checkpoints& ck, int* ns, int* mt, s
 // Vh_p: the packed V_h map with boxes of rpg rows; U64: U as 32-term boxes of
 // 128 rows with 64-byte swizzling.
 cudaError_t launch_tc_seq(const TcMap& Vh_p, const TcMap& U64, const TcSeqArgs& a, int ns, int mt, cudaStream_t s);
+
+// All T timesteps of a layer in one launch over all stream tiles, factors
+// resident on chip, h and tau' exchanged through L2 (k_tensor_loop.cu).
+constexpr int kLoopMaxTiles = 256;   // stream tiles (counters) of one launch
+struct TcLoopPlan {
+  int nt;                    // streams per tile
+  int ST;                    // stream tiles
+  int cs, ctas;              // CTAs per cluster, CTAs in the grid
+  int rpg, ktiles, RT;       // packed V_h rows per gate of a row tile (16, 32, 64, 128), 128-row tiles per gate, row tiles
+  int ga, nka, sa, nA;       // role A: CTAs that split H, 64-column chunks each, stream tiles per CTA, CTAs
+  int gp, UT, sb, nB;        // role B: gates per CTA, unit tiles, stream tiles per CTA, CTAs
+  int ures, ux_chunks;       // 64-term chunks of U per gate in tensor memory; chunks in shared memory
+  int acc_a, acc_b;          // tensor-memory columns of the accumulators of either role (U starts at column 0)
+  int shared_acc;            // 1: the two roles' accumulators share their columns
+  int ra_regions, rb_regions;  // accumulators of either role (its stream tiles take them in turn)
+  int defer_depths;          // 1: a step's intermediate depths run while the next step's tau' is on its way
+  int mb;                    // role B: both planes in one MMA (separate accumulators)
+  int share_rx;              // the roles' exchanges share their receive buffers
+  uint32_t rxa_bytes, rxb_bytes;
+  int stages;                // ring stages of 64 elements x nt streams x 2 planes
+  uint32_t smem;
+  int ncut;                  // intermediate depths below K
+};
+struct TcLoopArgs : TcLoopPlan {
+  int H, K, Ks, B, T;
+  int vbox;                  // rows of a V_h box
+  const __nv_bfloat16* U;    // [4][H][Ks]
+  const float* P;            // [T*B][ldp] hoisted input projection, column g*Ks + k
+  int ldp;
+  const float* sigma;
+  const float* bias;
+  const float* h0;           // [B][H] or null (zero)
+  const float* c0;
+  float* c_state;            // [B][H] scratch: c_t for odd and even t
+  float* c_state1;
+  __nv_bfloat16* h_bf16;     // pair planes [2][B][ldh]
+  int ldh;
+  long long h_plane;
+  __nv_bfloat16* tau;        // pair planes [2][B][ldt]
+  int ldt;
+  long long tau_plane;
+  float* out_h;              // [T][B][H] or null
+  float* c_last;             // [B][H] or null
+  __nv_bfloat16* seq_bf16;   // pair of h_t for the next layer: (t*B + n)*ldh + unit, lo plane at + seq_plane; or null
+  long long seq_plane;
+  int ck_n;
+  int cut_k[kMaxCheckpoints];
+  float* ckpt_h;             // element (j, t, n, unit) at j*ck_stride + (t*B + n)*H + unit, or null
+  float* ckpt_c;
+  long long ck_stride;
+  unsigned* h_count;         // one per stream tile, 32 words apart; zero before and after a launch
+  unsigned* tau_count;
+  unsigned* done;
+  int* err;
+  long long limit_ns;
+  int test_stall;            // 1: CTA 0 withholds its first h (the waits run out)
+};
+// Whether a layer of this shape takes the resident-factor launch, and how.
+bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out);
+// V: the V_h map whose boxes have a.vbox rows; U: U in boxes of 128 rows; Hm, Taum: h and tau' as planes
+// (tc_make_map_planes, boxes of p.nt rows).  *resident = false (and nothing launched) if the device
+// cannot hold the whole grid at once.
+cudaError_t launch_tc_loop(const TcMap& V, const TcMap& U, const TcMap& Hm, const TcMap& Taum, const TcLoopPlan& p,
+                           const TcLoopArgs& args, cudaStream_t s, bool* resident);
+// 3-D bf16 tensor [2 planes][rows][inner], boxes of 64 inner elements x box_rows rows x both planes, 128-byte swizzling.
+bool tc_make_map_planes(TcMap* m, const void* base, uint64_t inner, uint64_t rows, uint64_t pitch_bytes,
+                        uint64_t plane_bytes, uint32_t box_rows);
 
 // Compressed tau' (the recurrent part of the pruned v as (column, value)
 // entries per storage row g*Ks + k, entries off[row] .. off[row + 1]) on the

@@ -1019,6 +1019,22 @@ bool tc_make_map_f32(TcMap* m, const void* base, uint64_t inner, uint64_t rows, 
   return r == CUDA_SUCCESS;
 }
 
+bool tc_make_map_planes(TcMap* m, const void* base, uint64_t inner, uint64_t rows, uint64_t pitch_bytes,
+                        uint64_t plane_bytes, uint32_t box_rows) {
+  EncodeTiled enc = encoder();
+  if (!enc) return false;
+  std::memset(m->bytes, 0, sizeof(m->bytes));
+  const cuuint64_t dims[3] = {inner, rows, 2};
+  const cuuint64_t strides[2] = {pitch_bytes, plane_bytes};
+  const cuuint32_t box[3] = {64u, box_rows, 2u};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = enc(reinterpret_cast<CUtensorMap*>(m->bytes), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+                         const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 cudaError_t launch_tc_rows(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, int n_cols, int bn, cudaStream_t s) {
   switch (bn) {
     case 128: return launch_rows_t<128, 4>(A, Bm, a, n_cols, s);

@@ -437,9 +437,66 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
     LA_CUDA(h, launch_tc_seq(s.map_vh_p[pi], s.map_u64, qa, ns, utiles, h->stream), "recurrence launch");
     h->launches += 1;
     h->last_tensor_seq = 1;
+    h->last_tensor_loop = 0;
     return LSTM_APPROX_OK;
   }
   h->last_tensor_seq = 0;
+  TcLoopPlan lp;
+  if (h->opt_tensor_seq == 0 && h->opt_tau_layout == 0 && tc_loop_plan(H, B, K, ck, &lp)) {
+    // one launch over all stream tiles for all T timesteps, the factors resident (offsets within a
+    // timestep's P are 32-bit there: B * ldp below 2^31 follows from its limits on B and K)
+    TcMap mh, mt;
+    if (!tc_make_map_planes(&mh, hb, H, B, (uint64_t)h->ldh * 2, (uint64_t)B * h->ldh * 2, lp.nt) ||
+        !tc_make_map_planes(&mt, tau, ldp, B, (uint64_t)ldp * 2, (uint64_t)B * ldp * 2, lp.nt))
+      return fail(h, LSTM_APPROX_ECUDA, "tensor map encoding failed for the state");
+    TcLoopArgs qa{};
+    qa.H = H;
+    qa.K = K;
+    qa.Ks = h->Ks;
+    qa.B = B;
+    qa.T = T;
+    qa.vbox = lp.rpg == 128 ? 128 : lp.rpg == 16 ? 16 : 32;
+    qa.U = static_cast<const __nv_bfloat16*>(s.U);
+    qa.P = h->Px;
+    qa.ldp = (int)ldp;
+    qa.sigma = s.sigma;
+    qa.bias = s.bias;
+    qa.h0 = h0;
+    qa.c0 = c0;
+    qa.c_state = cs;
+    qa.c_state1 = h->h_state + (size_t)l * h->max_batch * H;  // (this path keeps h as its pair)
+    qa.h_bf16 = hb;
+    qa.ldh = h->ldh;
+    qa.h_plane = (long long)B * h->ldh;
+    qa.tau = tau;
+    qa.ldt = (int)ldp;
+    qa.tau_plane = (long long)B * ldp;
+    qa.out_h = out_h;
+    qa.c_last = out_c;
+    qa.seq_bf16 = top ? nullptr : static_cast<__nv_bfloat16*>(h->seq_bf16);
+    qa.seq_plane = (long long)TB * h->ldh;
+    qa.ck_n = ck.n;
+    for (int j = 0; j < ck.n; ++j) qa.cut_k[j] = ck.k[j];
+    qa.ckpt_h = ckpt_h;
+    qa.ckpt_c = ckpt_c;
+    qa.ck_stride = (long long)T * B * H;
+    qa.h_count = h->loop_counts;
+    qa.tau_count = h->loop_counts + 32 * kLoopMaxTiles;
+    qa.done = h->loop_counts + 64 * kLoopMaxTiles;
+    qa.err = h->err;
+    qa.limit_ns = limit_ns;
+    qa.test_stall = h->opt_test_stall;
+    bool resident = false;
+    const TcMap& mv = lp.rpg == 128 ? s.map_vh : s.map_vh_p[lp.rpg == 16 ? 1 : 2];
+    LA_CUDA(h, launch_tc_loop(mv, s.map_u, mh, mt, lp, qa, h->stream, &resident), "recurrence launch");
+    if (resident) {
+      h->opt_test_stall = 0;
+      h->launches += 1;
+      h->last_tensor_loop = 1;
+      return LSTM_APPROX_OK;
+    }
+  }
+  h->last_tensor_loop = 0;
   LA_CUDA(h, launch_tc_init_state(h0, c0, B, H, hb, h->ldh, cs, h->stream), "state init launch");
   h->launches += 1;
   // packed gates write only the first rpg terms of each gate's tau' rows; the
@@ -824,8 +881,10 @@ int lstm_approx_create(lstm_approx_t** out, int num_layers, const int* input_dim
   if (!rc) rc = dmalloc(h, reinterpret_cast<void**>(&h->c_state), state, "state");
   if (!rc) rc = dmalloc(h, &h->tau, (size_t)max_batch * 4 * h->Ks * sizeof(float), "scratch tau");
   if (!rc) rc = dmalloc(h, reinterpret_cast<void**>(&h->err), sizeof(int), "status word");
-  if (!rc)
-    rc = dmalloc(h, reinterpret_cast<void**>(&h->proj_flags), kProjFlags * sizeof(unsigned), "projection flags");
+  // completion flags of the projection, and on the tensor path the stream tiles' counters after them
+  const size_t flags = kProjFlags + (dtype == LSTM_APPROX_BF16 ? 64 * kLoopMaxTiles + 32 : 0);
+  if (!rc) rc = dmalloc(h, reinterpret_cast<void**>(&h->proj_flags), flags * sizeof(unsigned), "flags and counters");
+  if (!rc && dtype == LSTM_APPROX_BF16) h->loop_counts = h->proj_flags + kProjFlags;
   if (!rc && cudaHostAlloc(reinterpret_cast<void**>(&h->err_host), sizeof(int), cudaHostAllocDefault) != cudaSuccess)
     rc = fail(h, LSTM_APPROX_ENOMEM, "pinned status word");
   if (!rc && dtype == LSTM_APPROX_BF16)
@@ -1172,6 +1231,7 @@ int lstm_approx_query(const lstm_approx_t* h, int key, long long* value) {
     case LSTM_APPROX_Q_DEVICE_BYTES: *value = h->device_bytes; return LSTM_APPROX_OK;
     case LSTM_APPROX_Q_PERSISTENT_VARIANT: *value = h->last_variant; return LSTM_APPROX_OK;
     case LSTM_APPROX_Q_TENSOR_SEQ: *value = h->last_tensor_seq; return LSTM_APPROX_OK;
+    case LSTM_APPROX_Q_TENSOR_LOOP: *value = h->last_tensor_loop; return LSTM_APPROX_OK;
     default: return LSTM_APPROX_EINVAL;
   }
 }
@@ -1302,6 +1362,8 @@ int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int* chec
       v[LSTM_APPROX_PLAN_GATE_TILE_STREAMS] = tt.nt;
       v[LSTM_APPROX_PLAN_GATE_SPLITS] = tt.ks;
       v[LSTM_APPROX_PLAN_TAU_SPLITS] = tt.sk;
+      TcLoopPlan lp;
+      v[LSTM_APPROX_PLAN_TENSOR_LOOP] = tc_loop_plan(hidden, B, K, ck, &lp) ? 1 : 0;
     }
   }
   for (int i = 0; i < n_out; ++i) out[i] = i < LSTM_APPROX_PLAN_ITEMS ? v[i] : 0;

@@ -1,0 +1,152 @@
+"""GPU parity of the tensor path's launch over all stream tiles and timesteps
+with the factors resident on chip (bf16 factors; k_tensor_loop.cu), and the
+rule that chooses it (CPU).
+
+Each GPU case is checked against the oracle on the factors as the library
+stores them, and against the two-launches-per-step kernels on the same inputs.
+The second bound, 4e-4 of the largest value, is derived: both form the same
+products of the same bf16 pairs (2^-17 relative each), K + H terms of fp32 sums
+in another order (relative 2^-24 each), over T steps of a contracting cell.
+"""
+import numpy as np
+import pytest
+
+from parity_util import BF16_TOL, assert_parity, oracle_run, run_gpu
+from paper_1905_00689_gb300 import (BF16, LSTMApprox, LSTMApproxError, OPT_TEST_STALL, OPT_WAIT_LIMIT, Q_TENSOR_LOOP,
+                                    Q_TENSOR_SEQ, plan)
+from workloads import draw_factor_set, draw_inputs
+
+
+def _gates(H, C, K, nz, seed):
+    gates = [draw_factor_set(H, C, K, nz, seed + g) for g in range(4)]
+    rng = np.random.default_rng(seed)
+    for g in gates:
+        g["bias"] = 0.2 * rng.standard_normal(H)
+    return gates
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,T,B,K,cps", [
+    (64, 3, 1, 1, []),                      # one term, one stream: 16 packed rows per gate
+    (72, 2, 17, 16, [16]),                  # the largest K of 16 rows; a depth at K
+    (301, 3, 33, 17, [1, 16]),              # odd H (a padding column), 32 rows; a depth of one term
+    (640, 2, 40, 33, [3, 9, 20]),           # 64 rows, H over two CTAs, two depths in one slice
+    (128, 4, 32, 64, []),                   # whole tiles
+    (512, 3, 65, 65, [64]),                 # 128 rows, a depth at a chunk boundary
+    (1000, 2, 31, 128, [17, 100]),          # largest K with all gates in a CTA
+    (512, 3, 33, 129, [128]),               # one gate per CTA: the gate exchange
+    (1100, 2, 20, 200, [5, 48, 199]),       # H over four CTAs, both exchanges
+    (1024, 2, 40, 512, [32, 511]),          # both exchanges, groups of two and four
+    (2048, 2, 64, 1024, [16, 64, 256, 1024]),  # terms of U in shared memory, several tiles per CTA
+    (256, 2, 300, 1000, []),                # many row tiles: several stream tiles per CTA
+])
+def test_small_shapes(cuda_device, H, T, B, K, cps):
+    D = 48
+    gates = _gates(H, D + H, K, min(60, D + H), 8100 + H + K)
+    rng = np.random.default_rng(B)
+    x = draw_inputs(T, B, D, "uniform", 80 + B)
+    h0 = 0.3 * rng.standard_normal((1, B, H))
+    c0 = 0.3 * rng.standard_normal((1, B, H))
+    got, m = run_gpu([gates], x, K, dtype="bf16", h0=h0, c0=c0, checkpoints=cps)
+    assert m.query(Q_TENSOR_LOOP) == 1 == plan(BF16, H, T, B, K, cps)["tensor_loop"]
+    step, m2 = run_gpu([gates], x, K, dtype="bf16", h0=h0, c0=c0, checkpoints=cps, tensor_seq=1)
+    assert m2.query(Q_TENSOR_LOOP) == 0
+    for k in got:
+        assert np.abs(got[k] - step[k]).max() <= 4e-4 * np.abs(step[k]).max(), k
+    streams = sorted({0, B // 2, B - 1})
+    ref = oracle_run([gates], x[:, streams], K, dtype="bf16", h0=h0[:, streams], c0=c0[:, streams], checkpoints=cps)
+    cut = {k: v[:, streams] if k in ("h", "c_last") else v[:, :, streams] for k, v in got.items()}
+    assert_parity(cut, ref, BF16_TOL)
+
+
+@pytest.mark.gpu
+def test_two_layers_and_graph_replay(cuda_device):
+    """Layer 0 hands its sequence on as the pair; a captured run replayed on
+    new inputs equals an eager one (the counters are left at zero)."""
+    import torch
+    D, H, T, B, K = 72, 136, 4, 40, 48
+    layers = [_gates(H, (D if l == 0 else H) + H, K, 60, 8300 + 10 * l) for l in range(2)]
+    x = draw_inputs(T, B, D, "uniform", 83)
+    got, m = run_gpu(layers, x, K, dtype="bf16", checkpoints=[10])
+    assert m.query(Q_TENSOR_LOOP) == 1
+    assert_parity(got, oracle_run(layers, x, K, dtype="bf16", checkpoints=[10]), BF16_TOL)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        m = LSTMApprox(2, [D, H], H, K, B, "bf16", stream=s)
+        for l in range(2):
+            m.set_layer(l, layers[l])
+        xt = torch.zeros(T, B, D, device="cuda")
+        out = torch.empty(T, B, H, device="cuda")
+        m.run(xt, K, out)
+        m.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            m.run(xt, K, out)
+        xt.copy_(torch.from_numpy(x.astype(np.float32)))
+        for _ in range(2):
+            g.replay()
+        m.sync()
+    eager, _ = run_gpu(layers, x, K, dtype="bf16")  # the same call: no depths, so the same order of sums
+    assert np.array_equal(out.double().cpu().numpy(), eager["h"])
+
+
+@pytest.mark.gpu
+def test_two_handles_on_two_streams(cuda_device):
+    """Launches of two handles on two streams, each needing most of the SMs
+    at once, complete and agree."""
+    import torch
+    D, H, T, B, K = 64, 512, 6, 256, 200
+    gates = _gates(H, D + H, K, 100, 8400)
+    x = torch.from_numpy(draw_inputs(T, B, D, "uniform", 84).astype(np.float32)).cuda()
+    runs = []
+    for _ in range(2):
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            m = LSTMApprox(1, [D], H, K, B, "bf16", stream=s)
+            m.set_layer(0, gates)
+            runs.append((s, m, torch.empty(T, B, H, device="cuda")))
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for s, m, out in runs:
+            with torch.cuda.stream(s):
+                m.run(x, K, out)
+    for s, m, out in runs:
+        m.sync()
+        assert m.query(Q_TENSOR_LOOP) == 1
+    assert torch.equal(runs[0][2], runs[1][2])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,K", [(136, 40), (1024, 200)])
+def test_bounded_wait_reports_timeout(cuda_device, H, K):
+    """CTA 0 withholds its first h: the waits run out after the short limit,
+    the run reports ETIMEOUT, and the next run on the handle is correct."""
+    import torch
+    D, T, B = 32, 3, 20
+    gates = _gates(H, D + H, K, 40, 8500)
+    x = draw_inputs(T, B, D, "uniform", 85)
+    ref, m = run_gpu([gates], x, K, dtype="bf16")
+    m.set_option(OPT_WAIT_LIMIT, 50_000)  # 50 ms
+    m.set_option(OPT_TEST_STALL, 1)
+    xt = torch.from_numpy(x.astype(np.float32)).cuda()
+    out = torch.zeros((T, B, H), device="cuda")
+    m.run(xt, K, out)
+    with pytest.raises(LSTMApproxError) as ei:
+        m.sync()
+    assert ei.value.code == 4  # LSTM_APPROX_ETIMEOUT
+    m.set_option(OPT_WAIT_LIMIT, 2_000_000)
+    m.run(xt, K, out)
+    m.sync()
+    assert np.array_equal(out.double().cpu().numpy(), ref["h"])
+
+
+@pytest.mark.parametrize("H,B,K,cps,loop", [
+    (512, 256, 512, [], 1), (512, 256, 32, [], 0),             # K <= 32 at H = 512: one launch per stream tile
+    (600, 100, 32, [10], 1), (2048, 64, 1024, [16, 256], 1),
+    (2049, 16, 64, [], 0), (2048, 16, 1025, [], 0),             # outside its limits
+    (1024, 1024, 128, [], 1), (1024, 1024, 512, [], 0),         # too many streams per CTA
+])
+def test_rule(H, B, K, cps, loop):
+    p = plan(BF16, H, 2, B, K, cps)
+    assert p["tensor_loop"] == loop
+    assert p["tensor_seq"] == (1 if K <= 32 and H == 512 else 0)
