@@ -167,36 +167,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8]) {
                : "memory");
 }
 
-// One poll of an mbarrier phase with a suspend-time hint, so that a waiting warp sleeps instead of taking
-// issue slots from the threads that issue the copies and MMAs on its scheduler.
-template <bool kCluster>
-__device__ __forceinline__ bool poll(uint32_t mb, uint32_t parity) {
-  if constexpr (kCluster) {
-    return mbar_try_wait_cluster(mb, parity) != 0u;
-  } else {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(mb), "r"(parity), "r"(20000u)
-        : "memory");
-    return ok != 0u;
-  }
-}
-// Bounded wait on an mbarrier phase, as mbar_wait_bounded in fewer instructions.
-template <bool kCluster>
-__device__ __forceinline__ bool loop_wait(uint32_t mb, uint32_t parity, uint64_t limit_ns, const volatile int* err) {
-  if (poll<kCluster>(mb, parity)) return true;
-  const uint64_t t0 = global_timer_ns();
-  do {
-#pragma unroll 1
-    for (int i = 0; i < 8; ++i)
-      if (poll<kCluster>(mb, parity)) return true;
-  } while (*err == 0 && global_timer_ns() - t0 <= limit_ns);
-  return false;
-}
-
 // Bounded wait until *c has reached `target` (acquire at GPU scope), then
 // orders later TMA reads of this thread after what the counter released.
 __device__ __forceinline__ bool wait_counter(const unsigned* c, unsigned target, uint64_t limit,
@@ -329,7 +299,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       RingPos pos;
       auto load = [&](const CUtensorMap* m, int c0, int row) {
         // the slot's previous load (one ring round ago) has been consumed
-        if (it == stages && !(ok = loop_wait<false>(empty0 + 8u * pos.slot, pos.parity ^ 1u, limit, err))) return;
+        if (it == stages && !(ok = mbar_wait_bounded<false>(empty0 + 8u * pos.slot, pos.parity ^ 1u, limit, err))) return;
         const uint32_t bar_s = full0 + 8u * pos.slot;
         mbar_arrive_expect_tx(bar_s, kStage);
         tma_load_3d(base + L.ring + pos.slot * kStage, m, bar_s, c0, row, 0);
@@ -354,15 +324,15 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       }
       if (!ok) atomicCAS(a.err, 0, kErrTcTimeout);
       // every issued copy has landed before the CTA may leave
-      loop_wait<false>(setup_bar, 0, limit, err);
+      mbar_wait_bounded<false>(setup_bar, 0, limit, err);
       for (int s = 0; s < it; ++s)  // slot s was last filled in this round (before the position) or the one before
-        loop_wait<false>(full0 + 8u * s, s < pos.slot ? pos.parity : pos.parity ^ 1u, limit, err);
+        mbar_wait_bounded<false>(full0 + 8u * s, s < pos.slot ? pos.parity : pos.parity ^ 1u, limit, err);
     }
   } else if (warp == 1) {
     if (elect_one()) {  // ---- MMA issuer ----
       constexpr uint32_t idesc2 = umma_idesc_bf16(128, 2 * NT);
       constexpr uint32_t idesc_b = umma_idesc_bf16(128, MB ? 2 * NT : NT);
-      bool ok = loop_wait<false>(setup_bar, 0, limit, err) && loop_wait<false>(u_ready, 0, limit, err);
+      bool ok = mbar_wait_bounded<false>(setup_bar, 0, limit, err) && mbar_wait_bounded<false>(u_ready, 0, limit, err);
       tc_fence_after();
       const int stages = a.stages;
       RingPos pos;
@@ -375,12 +345,12 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           ++used;
           return true;
         }
-        return loop_wait<false>(bars + 8u * p.slot, p.parity ^ 1u, limit, err);
+        return mbar_wait_bounded<false>(bars + 8u * p.slot, p.parity ^ 1u, limit, err);
       };
       // the other role's accumulators in the same columns: its last item so far has been read
       auto last_drained = [&](uint32_t bars, const RingPos& p, int regions) {
         const int slot = p.slot == 0 ? regions - 1 : p.slot - 1;
-        return loop_wait<false>(bars + 8u * slot, p.slot == 0 ? p.parity ^ 1u : p.parity, limit, err);
+        return mbar_wait_bounded<false>(bars + 8u * slot, p.slot == 0 ? p.parity ^ 1u : p.parity, limit, err);
       };
       constexpr uint32_t dg = NT * (MB ? 2 : 1);  // columns of one gate's accumulator
       constexpr uint32_t seg = GP * dg;           // of one depth segment
@@ -407,7 +377,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           uint32_t acc = 0;
 #pragma unroll 1
           for (int c = 0; c < nkh; ++c) {
-            if (!(ok = loop_wait<false>(full0 + 8u * pos.slot, pos.parity, limit, err))) break;
+            if (!(ok = mbar_wait_bounded<false>(full0 + 8u * pos.slot, pos.parity, limit, err))) break;
             tc_fence_after();
             const uint64_t db = ring_desc + (uint64_t)((uint32_t)pos.slot * (kStage >> 4));
 #pragma unroll
@@ -438,7 +408,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
             uint32_t freed[GP];  // the empty barriers of this chunk's slots
 #pragma unroll
             for (int g = 0; g < GP; ++g) {
-              ok = ok && loop_wait<false>(full0 + 8u * pos.slot, pos.parity, limit, err);
+              ok = ok && mbar_wait_bounded<false>(full0 + 8u * pos.slot, pos.parity, limit, err);
               db[g] = ring_desc + (uint64_t)((uint32_t)pos.slot * (kStage >> 4));
               freed[g] = empty0 + 8u * pos.slot;
               pos.next(stages);
@@ -492,7 +462,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       }
       if (!ok) atomicCAS(a.err, 0, kErrTcTimeout);
       umma_commit(final_bar);  // every MMA issued has completed before tensor memory is freed
-      loop_wait<false>(final_bar, 0, limit, err);
+      mbar_wait_bounded<false>(final_bar, 0, limit, err);
     }
   } else {  // ---- epilogue ----
     const int e = threadIdx.x - 64, q = warp & 3, part = (warp - 2) >> 2;
@@ -700,7 +670,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           tc_fence_before();
           warp_arrive(drain_b + 8u * region);
         }
-        const bool got = __all_sync(0xffffffffu, loop_wait<true>(rxb, (u >> 1) & 1u, limit, err));
+        const bool got = __all_sync(0xffffffffu, mbar_wait_bounded<true>(rxb, (u >> 1) & 1u, limit, err));
         const float* rb = reinterpret_cast<const float*>(gb_ + buf) + part * CPT;
 #pragma unroll
         for (int g = 0; g < 4; ++g)
@@ -808,7 +778,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           const int n = n0 + fc0 + c;
           pv[c] = (c < fcn && fr.valid && n < B) ? __ldg(Pt + n * a.ldp) : 0.f;
         }
-        bool fail = !__all_sync(0xffffffffu, loop_wait<false>(acc_a + 8u * pa.slot, pa.parity, limit, err));
+        bool fail = !__all_sync(0xffffffffu, mbar_wait_bounded<false>(acc_a + 8u * pa.slot, pa.parity, limit, err));
         const uint32_t handed = drain_a + 8u * pa.slot;
         if (!fail) {
           tc_fence_after();
@@ -858,7 +828,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
                             vh[4 * h4 + 1] + vl[4 * h4 + 1], vh[4 * h4 + 2] + vl[4 * h4 + 2],
                             vh[4 * h4 + 3] + vl[4 * h4 + 3], dbar);
             }
-            fail = !__all_sync(0xffffffffu, loop_wait<true>(rxb, (u >> 1) & 1u, limit, err));
+            fail = !__all_sync(0xffffffffu, mbar_wait_bounded<true>(rxb, (u >> 1) & 1u, limit, err));
             if (!fail) {
               // the group's partial sums in rank order (the result does not depend on timing)
               const uint8_t* rb = gb_ + buf;
@@ -889,7 +859,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
 #pragma unroll 1
       for (int s = 0; s < nb && ok; ++s) {
         if (t == 0 || !keep_c) load_c(t, first_stream(s));
-        const bool got = __all_sync(0xffffffffu, loop_wait<false>(acc_b + 8u * pb.slot, pb.parity, limit, err));
+        const bool got = __all_sync(0xffffffffu, mbar_wait_bounded<false>(acc_b + 8u * pb.slot, pb.parity, limit, err));
         tc_fence_after();
         bool good = got && run_sets(t, s, pb.slot, 0, 1);
         if (!got) good = publish(true, a.h_count, true);

@@ -83,10 +83,10 @@ __device__ __forceinline__ uint32_t mbar_try_wait_cta(uint32_t mb, uint32_t pari
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(mb), "r"(parity)
+      : "r"(mb), "r"(parity), "r"(20000u)
       : "memory");
   return ok;
 }
@@ -97,15 +97,15 @@ __device__ __forceinline__ uint32_t mbar_try_wait_cta(uint32_t mb, uint32_t pari
 template <bool kCluster>
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mb, uint32_t parity, uint64_t limit_ns,
                                                   const volatile int* err) {
-  if (kCluster ? mbar_try_wait_cluster(mb, parity) : mbar_try_wait_cta(mb, parity)) return true;
+  auto poll = [&]() { return kCluster ? mbar_try_wait_cluster(mb, parity) : mbar_try_wait_cta(mb, parity); };
+  if (poll()) return true;
   const uint64_t t0 = global_timer_ns();
-  for (uint32_t i = 1;; ++i) {
-    if (kCluster ? mbar_try_wait_cluster(mb, parity) : mbar_try_wait_cta(mb, parity)) return true;
-    if ((i & 15u) == 0u) {
-      if (*err != 0) return false;
-      if (global_timer_ns() - t0 > limit_ns) return false;
-    }
-  }
+  do {
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i)
+      if (poll()) return true;
+  } while (*err == 0 && global_timer_ns() - t0 <= limit_ns);
+  return false;
 }
 
 // 16-byte store into (possibly remote) shared memory of the cluster, which
