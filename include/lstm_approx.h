@@ -264,7 +264,8 @@ enum lstm_approx_query_key {
   LSTM_APPROX_Q_CLUSTER = 2,     /* CTAs per cluster of the last persistent run */
   LSTM_APPROX_Q_DEVICE_BYTES = 3, /* device bytes currently held by the handle */
   LSTM_APPROX_Q_PERSISTENT_VARIANT = 4, /* persistent kernel of the last persistent run
-                                          (1 or 2, see LSTM_APPROX_OPT_PERSISTENT_VARIANT) */
+                                          (1 or 2, see LSTM_APPROX_OPT_PERSISTENT_VARIANT, or
+                                          3: one CTA per stream, automatic only) */
   LSTM_APPROX_Q_TENSOR_SEQ = 5,  /* 1 if the last tensor-path layer ran as one launch per
                                     stream tile for all timesteps (see LSTM_APPROX_OPT_TENSOR_SEQ) */
   LSTM_APPROX_Q_TENSOR_LOOP = 6  /* 1 if it ran as one launch over all stream tiles for all
@@ -389,7 +390,11 @@ enum lstm_approx_plan_item {
                                               T (the tile and split items then describe the
                                               per-timestep kernels that serve where the device cannot
                                               hold that launch at once) */
-  LSTM_APPROX_PLAN_ITEMS = 16
+  LSTM_APPROX_PLAN_ONE_CTA = 16,           /* persistent path: 1 = a run with no forced path, cluster, kernel or
+                                              projection takes one CTA per stream with the factors in registers
+                                              (LSTM_APPROX_Q_PERSISTENT_VARIANT 3) instead of the cluster kernel
+                                              that the other items describe */
+  LSTM_APPROX_PLAN_ITEMS = 17
 };
 int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int *checkpoints, int J,
                      int force_path, int cluster, int persistent_variant, int *out, int n_out,

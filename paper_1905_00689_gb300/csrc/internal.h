@@ -248,6 +248,27 @@ bool plan_persistent_ag(int H, int K, const Checkpoints& ck, int want_cs, Persis
                         std::string* why);
 cudaError_t launch_persistent_ag(const PersistentAgPlan& plan, const PersistentArgs& a, cudaStream_t s);
 
+// One CTA per stream, the factors in its registers (H, K <= 128 and few
+// values per thread), with the input projection inside where it is small.
+struct PersistentOnePlan {
+  int threads = 0;     // 128, 256 or 512
+  int LA = 0, LB = 0;  // lanes per coefficient row, per gate row
+  int VQ = 0;          // quads of either factor per thread (1, 2, 4 or 8)
+  int HP = 0, KP = 0;  // shared-memory strides of h and of a gate's tau'
+};
+struct OneProj {
+  int mode = 0;             // 0: P comes from an earlier launch; 1: dense rows of Vx; 2: compressed rows
+  const float* x = nullptr;  // [T][B][D]
+  int D = 0;
+  const float* Vx = nullptr;  // [4*Ks][ldx]
+  int ldx = 0;
+  SparseXRows sparse{};
+};
+bool plan_persistent_one(int H, int K, bool gathers, PersistentOnePlan* out);  // gathers: OneProj mode 2
+int persistent_one_projection(int K, int T, int D, long long kept_x, bool sparse);
+cudaError_t launch_persistent_one(const PersistentOnePlan& p, const PersistentArgs& a, const OneProj& pr,
+                                  cudaStream_t s);
+
 // Either persistent kernel: variant 1 = per-unit-block kernel (two
 // exchanges per step), 2 = one-exchange kernel; 0 picks the one-exchange
 // kernel where it fits and a CTA's share (H x terms per CTA) is small, else

@@ -181,6 +181,8 @@ void clear_timing(lstm_approx_t* h) {
   h->timing.phase.clear();
 }
 
+constexpr int kOneProjMaxStreams = 152;  // one CTA per SM
+
 // The compressed x projection pays when v keeps at most 1/8 of the x columns
 // (fp32 factors, few columns).
 bool sparse_x_projection(const lstm_approx_t* h, const LayerStore& s, int K, int N) {
@@ -675,6 +677,34 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
     // faster although the projection takes 15.8 instead of 10.5 us).
     // Shorter set-ups gain less than the slower projection costs (K = 64: 4%
     // slower, the one-exchange kernel at K = 16: 11%).
+    // One stream's factors in one CTA's registers: nothing is exchanged, and a small projection runs inside
+    // (D = 64, H = 64, T = 8, K = 16, one stream: 24.2 -> 10.7 us a call; the case-study shape, D = 8256, H = 64, T = 1,
+    // K = 16 at 130 kept entries: 8.2 -> 5.8 us).  Forced kernels, clusters and projections take the others.
+    PersistentOnePlan one;
+    const bool use_one = path == LSTM_APPROX_PATH_PERSISTENT && h->opt_force_path == 0 && h->opt_cluster == 0 &&
+                         h->opt_persistent_variant == 0 && h->opt_xproj == 0 && h->opt_test_stall == 0 &&
+                         plan_persistent_one(H, K, false, &one);
+    OneProj one_proj;
+    if (use_one && B <= kOneProjMaxStreams) {  // every CTA reads the projection's rows: not for many streams
+      long long kept = 0;
+      bool have = true;
+      for (int g = 0; g < 4; ++g) {
+        have = have && s.xoff[g] != nullptr && (int)s.xoff_h[g].size() > K;
+        if (have) kept += s.xoff_h[g][K];
+      }
+      const bool sp = have && kept * 8 <= 4LL * K * s.D;
+      one_proj.mode = persistent_one_projection(K, T, s.D, kept, sp);
+      one_proj.x = in;
+      one_proj.D = s.D;
+      one_proj.Vx = static_cast<const float*>(s.Vx);
+      one_proj.ldx = s.ldx;
+      for (int g = 0; g < 4; ++g) {
+        one_proj.sparse.off[g] = s.xoff[g];
+        one_proj.sparse.idx[g] = s.xidx[g];
+        one_proj.sparse.val[g] = s.xval[g];
+      }
+      if (one_proj.mode == 2 && !plan_persistent_one(H, K, true, &one)) one_proj.mode = 0;
+    }
     const bool sparse_x = sparse_x_projection(h, s, K, T * B);
     const bool cluster_x = !sparse_x && xproj_cluster_fits(T * B, s.D, s.Vx, s.ldx, in, s.D, bf16);
     // (not while the stream is being captured: a graph would replay the
@@ -682,13 +712,13 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
     // previous replay would already hold it)
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess) capture = cudaStreamCaptureStatusActive;
-    bool rec_first = path == LSTM_APPROX_PATH_PERSISTENT && plan.variant == 1 && B == 1 && cluster_x &&
+    bool rec_first = path == LSTM_APPROX_PATH_PERSISTENT && !use_one && plan.variant == 1 && B == 1 && cluster_x &&
                      !h->timing.on && h->opt_launch_order == 0 && h->proj_flags != nullptr &&
                      capture == cudaStreamCaptureStatusNone;
     const int proj_ctas = rec_first ? xproj_cluster_ctas(K, T * B, s.D, 8) : 0;
     rec_first = rec_first && proj_ctas <= kProjFlags && xproj_cluster_prepare(bf16, T * B) == cudaSuccess;
     const int xproj_max_split =
-        rec_first ? 8 : (path == LSTM_APPROX_PATH_PERSISTENT && plan.variant == 1 && K > 128) ? 1 : 8;
+        rec_first ? 8 : (path == LSTM_APPROX_PATH_PERSISTENT && !use_one && plan.variant == 1 && K > 128) ? 1 : 8;
     XprojSignal sig;
     if (rec_first) {
       if (++h->proj_epoch == 0) ++h->proj_epoch;  // the flags start at zero
@@ -720,7 +750,7 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
       h->launches += 1;
       return LSTM_APPROX_OK;
     };
-    if (!rec_first) {
+    if (!rec_first && one_proj.mode == 0) {
       rc = launch_projection();
       if (rc) return rc;
     }
@@ -754,10 +784,13 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
         a.proj_epoch = sig.epoch;
       }
       h->opt_test_stall = 0;
-      LA_CUDA(h, launch_persistent_choice(plan, a, h->stream), "persistent kernel launch");
+      if (use_one)
+        LA_CUDA(h, launch_persistent_one(one, a, one_proj, h->stream), "persistent kernel launch");
+      else
+        LA_CUDA(h, launch_persistent_choice(plan, a, h->stream), "persistent kernel launch");
       h->launches += 1;
-      h->last_cluster = plan.CS;
-      h->last_variant = plan.variant;
+      h->last_cluster = use_one ? 1 : plan.CS;
+      h->last_variant = use_one ? 3 : plan.variant;
       if (rec_first) {
         rc = launch_projection();
         if (rc) return rc;
@@ -1347,6 +1380,8 @@ int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int* chec
       v[LSTM_APPROX_PLAN_SMEM_BYTES] = (int)pc.ag.smem;
       v[LSTM_APPROX_PLAN_TMEM_COLUMNS] = pc.ag.tcols;
     }
+    PersistentOnePlan one;
+    v[LSTM_APPROX_PLAN_ONE_CTA] = plan_persistent_one(hidden, K, false, &one) ? 1 : 0;
   } else if (path == LSTM_APPROX_PATH_TENSOR) {
     int ns = 0, mt = 0;
     if (tc_seq_fits(hidden, B, K, ck, &ns, &mt, nullptr)) {
