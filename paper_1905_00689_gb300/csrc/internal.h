@@ -244,7 +244,7 @@ struct PersistentAgPlan {
   int hq = 0;       // h quads per lane in the recurrent product (1, 2 or 4)
   size_t smem = 0;  // dynamic shared memory bytes
 };
-bool plan_persistent_ag(int H, int K, const Checkpoints& ck, int want_cs, PersistentAgPlan* plan,
+bool plan_persistent_ag(int H, int K, int B, const Checkpoints& ck, int want_cs, PersistentAgPlan* plan,
                         std::string* why);
 cudaError_t launch_persistent_ag(const PersistentAgPlan& plan, const PersistentArgs& a, cudaStream_t s);
 
@@ -279,7 +279,7 @@ struct PersistentChoice {
   PersistentPlan ub;
   PersistentAgPlan ag;
 };
-bool choose_persistent(int H, int K, int T, const Checkpoints& ck, int want_cs, int sm_count, int variant,
+bool choose_persistent(int H, int K, int T, int B, const Checkpoints& ck, int want_cs, int sm_count, int variant,
                        PersistentChoice* c, std::string* why);
 cudaError_t launch_persistent_choice(const PersistentChoice& c, const PersistentArgs& a, cudaStream_t s);
 

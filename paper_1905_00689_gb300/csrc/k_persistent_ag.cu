@@ -454,7 +454,13 @@ __global__ void __launch_bounds__(kThreads, 1) persistent_ag_kernel(PersistentAr
 }
 }  // namespace
 
-bool plan_persistent_ag(int H, int K, const Checkpoints& ck, int want_cs, PersistentAgPlan* plan,
+namespace {
+// Clusters of cs CTAs (one per SM) resident at once on a GB300: measured by the streams at which a second
+// wave starts.
+int resident_clusters(int cs) { return cs == 16 ? 7 : cs == 8 ? 15 : cs == 4 ? 36 : cs == 2 ? 76 : 152; }
+}  // namespace
+
+bool plan_persistent_ag(int H, int K, int B, const Checkpoints& ck, int want_cs, PersistentAgPlan* plan,
                         std::string* why) {
   if (H % 4 != 0 || H > kThreads) {
     *why = "hidden size not a multiple of 4 or above 512";
@@ -495,7 +501,15 @@ bool plan_persistent_ag(int H, int K, const Checkpoints& ck, int want_cs, Persis
     plan->tcols = p.tcols;
     plan->hq = hq;
     plan->smem = smem;
-    return true;  // the smallest cluster that fits moves the fewest partials
+    // the smallest cluster that fits moves the fewest partials, except that 48 or more terms per CTA take
+    // longer than the next size's extra partials (recurrence of 20 steps, clusters of 4 / 8: H = 200, K = 50
+    // 38.4 / 34.3 us, H = 256, K = 64 38.4 / 36.4; with 16 terms per CTA, H = 512, K = 16, 36.4 / 40.4)
+    PersistentAgPlan wider;
+    std::string unused;
+    if (want_cs == 0 && cs == 4 && p.RA >= 48 && H >= 128 && H <= 256 && B <= resident_clusters(8) &&
+        plan_persistent_ag(H, K, B, ck, 8, &wider, &unused))
+      *plan = wider;
+    return true;
   }
   *why = "shape does not fit the one-exchange persistent kernel (K, checkpoints or on-chip memory)";
   return false;
@@ -574,10 +588,13 @@ cudaError_t launch_persistent_ag(const PersistentAgPlan& plan, const PersistentA
 // sums 16 partial vectors of 512 floats per step.
 constexpr int kAgAutoMaxWork = 16384;
 
-bool choose_persistent(int H, int K, int T, const Checkpoints& ck, int want_cs, int sm_count, int variant,
-                       PersistentChoice* c, std::string* why) {
+namespace {
+
+// The kernel and cluster size of one wave's streams (a forced variant or cluster size is kept).
+bool choose_one_wave(int H, int K, int T, int B, const Checkpoints& ck, int want_cs, int sm_count, int variant,
+                     PersistentChoice* c, std::string* why) {
   std::string why_ag;
-  if (variant != 1 && plan_persistent_ag(H, K, ck, want_cs, &c->ag, &why_ag) &&
+  if (variant != 1 && plan_persistent_ag(H, K, B, ck, want_cs, &c->ag, &why_ag) &&
       (variant == 2 || H * c->ag.RA <= kAgAutoMaxWork)) {
     c->variant = 2;
     c->CS = c->ag.CS;
@@ -590,6 +607,31 @@ bool choose_persistent(int H, int K, int T, const Checkpoints& ck, int want_cs, 
   if (!plan_persistent(H, K, T, ck, want_cs, sm_count, &c->ub, why)) return false;
   c->variant = 1;
   c->CS = c->ub.CS;
+  return true;
+}
+
+}  // namespace
+
+bool choose_persistent(int H, int K, int T, int B, const Checkpoints& ck, int want_cs, int sm_count, int variant,
+                       PersistentChoice* c, std::string* why) {
+  if (!choose_one_wave(H, K, T, B, ck, want_cs, sm_count, variant, c, why)) return false;
+  if (variant != 0 || want_cs != 0 || B <= resident_clusters(c->CS)) return true;
+  // More streams than resident clusters: a second wave takes as long as the first, so a smaller cluster that
+  // holds them all is faster although its step is longer.  20 steps at H = 512, K = 64: 8 streams 73.2 us on
+  // clusters of 16, 40.4 on 8; 24 streams 140.8, 77.2, 50.7 (one-exchange kernel on 4); H = 256, K = 200, 8
+  // streams 85.5 (one-exchange, 16), 67.1 (8).  Relative time of a step by kernel and cluster size:
+  auto weight = [](int v, int cs) { return v == 1 ? (cs == 16 ? 10 : cs == 8 ? 11 : 13) : (cs == 8 ? 11 : 12); };
+  auto cost = [&](int v, int cs) { return (long long)((B + resident_clusters(cs) - 1) / resident_clusters(cs)) * weight(v, cs); };
+  long long best = cost(c->variant, c->CS);
+  for (int v : {1, 2})
+    for (int cs : {8, 4}) {
+      PersistentChoice alt;
+      std::string unused;
+      if (cost(v, cs) < best && choose_one_wave(H, K, T, B, ck, cs, sm_count, v, &alt, &unused)) {
+        *c = alt;
+        best = cost(v, cs);
+      }
+    }
   return true;
 }
 

@@ -205,13 +205,13 @@ bool tensor_path_fits(int dtype) { return dtype == LSTM_APPROX_BF16; }
 // clusters beyond one wave run in the next); everything else takes the
 // CUDA-core kernels.  A forced path that cannot take the shape returns 0
 // with the reason in *why.  *plan is filled for the persistent path.
-int select_path(int dtype, int H, int K, int T, const Checkpoints& ck, int force_path, int want_cs, int sm_count,
+int select_path(int dtype, int H, int K, int T, int B, const Checkpoints& ck, int force_path, int want_cs, int sm_count,
                 int variant, PersistentChoice* plan, std::string* why) {
   const bool bf16 = dtype == LSTM_APPROX_BF16;
   const bool tensor_ok = tensor_path_fits(dtype);
   if (force_path == 0) {
     if (tensor_ok) return LSTM_APPROX_PATH_TENSOR;
-    if (!bf16 && choose_persistent(H, K, T, ck, want_cs, sm_count, variant, plan, why))
+    if (!bf16 && choose_persistent(H, K, T, B, ck, want_cs, sm_count, variant, plan, why))
       return LSTM_APPROX_PATH_PERSISTENT;
     return LSTM_APPROX_PATH_SIMT;
   }
@@ -221,7 +221,7 @@ int select_path(int dtype, int H, int K, int T, const Checkpoints& ck, int force
       return 0;
     }
     std::string r;
-    if (!choose_persistent(H, K, T, ck, want_cs, sm_count, variant, plan, &r)) {
+    if (!choose_persistent(H, K, T, B, ck, want_cs, sm_count, variant, plan, &r)) {
       *why = "persistent path unavailable: " + r;
       return 0;
     }
@@ -626,7 +626,7 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
   if (bf16) {
     PersistentChoice unused;
     std::string why;
-    run_path = select_path(h->dtype, H, K, T, ck, h->opt_force_path, h->opt_cluster, h->sm_count,
+    run_path = select_path(h->dtype, H, K, T, B, ck, h->opt_force_path, h->opt_cluster, h->sm_count,
                            h->opt_persistent_variant, &unused, &why);
     if (run_path == 0) return fail(h, LSTM_APPROX_EINVAL, "%s", why.c_str());
   }
@@ -641,7 +641,7 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
     PersistentChoice plan;
     std::string why;
     const int path = bf16 ? run_path
-                          : select_path(h->dtype, H, K, T, lck, h->opt_force_path, h->opt_cluster, h->sm_count,
+                          : select_path(h->dtype, H, K, T, B, lck, h->opt_force_path, h->opt_cluster, h->sm_count,
                                         h->opt_persistent_variant, &plan, &why);
     if (path == 0) return fail(h, LSTM_APPROX_EINVAL, "%s", why.c_str());
     const float* l_h0 = h0 ? h0 + (size_t)l * B * H : nullptr;
@@ -1360,7 +1360,7 @@ int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int* chec
   if (n_out < 0 || (n_out > 0 && !out)) return report(msg, msg_len, E, "out is NULL with n_out=%d", n_out);
   PersistentChoice pc;
   std::string why;
-  const int path = select_path(dtype, hidden, K, T, ck, force_path, cluster, 0, persistent_variant, &pc, &why);
+  const int path = select_path(dtype, hidden, K, T, B, ck, force_path, cluster, 0, persistent_variant, &pc, &why);
   if (path == 0) return report(msg, msg_len, E, "%s", why.c_str());
   int v[LSTM_APPROX_PLAN_ITEMS] = {};
   v[LSTM_APPROX_PLAN_PATH] = path;

@@ -100,7 +100,7 @@ extern "C" int lstm_approx_run_static(const float* Vx, const float* Vh, const fl
 
   PersistentChoice plan;
   std::string why;
-  if (!choose_persistent(H, K, T, ck, 0, sms, 0, &plan, &why))
+  if (!choose_persistent(H, K, T, B, ck, 0, sms, 0, &plan, &why))
     return report(msg, msg_len, LSTM_APPROX_EINVAL, "shape does not fit: %s", why.c_str());
 
   float* base = nullptr;

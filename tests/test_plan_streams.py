@@ -1,0 +1,22 @@
+"""The persistent kernel and cluster size for several fp32 streams (host only):
+one cluster serves one stream, and clusters beyond those resident at once run
+in a second wave."""
+import pytest
+
+from paper_1905_00689_gb300 import FP32, plan
+
+RESIDENT = {16: 7, 8: 15, 4: 36}
+
+
+@pytest.mark.parametrize("H,K,B,variant,cluster", [
+    (512, 64, 7, 1, 16), (512, 64, 8, 1, 8), (512, 64, 15, 1, 8), (512, 64, 16, 2, 4), (512, 64, 36, 2, 4),
+    (512, 256, 8, 1, 16),                       # no smaller cluster holds it
+    (256, 200, 7, 2, 16), (256, 200, 8, 1, 8),
+    (200, 50, 15, 2, 8), (200, 50, 16, 2, 4),   # 48 terms per CTA or more: clusters of 8 up to one wave
+    (256, 32, 1, 2, 4), (512, 16, 30, 2, 4),
+])
+def test_streams_choose_the_cluster(H, K, B, variant, cluster):
+    p = plan(FP32, H, 20, B, K)
+    assert (p["persistent_variant"], p["cluster"]) == (variant, cluster)
+    if cluster < 16:
+        assert B <= RESIDENT[cluster]
