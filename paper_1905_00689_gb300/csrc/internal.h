@@ -132,8 +132,9 @@ cudaError_t launch_rows_gemm(const void* A, bool a_bf16, int lda, int K, int Ks,
 
 // Same product for few columns (N = T*B <= 256, in chunks of 32): clusters
 // split the D axis, rows are staged by asynchronous copies and the chunk
-// sums pushed to their owner CTA (deterministic).  Needs D % 8 == 0 and
-// 16-byte aligned base pointers and rows; a push that does not arrive
+// sums pushed to their owner CTA (deterministic).  Needs 16-byte aligned
+// rows of A, zero from D to a multiple of 4 (bf16 factors: D % 8 == 0 and
+// 16-byte aligned rows of X too); a push that does not arrive
 // within limit_ns sets *err.  max_split caps the CTAs per cluster along D
 // (1: one CTA per row tile and column chunk).
 bool xproj_cluster_fits(int N, int D, const void* A, int lda, const float* X, int ldxin, bool a_bf16);

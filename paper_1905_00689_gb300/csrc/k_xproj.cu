@@ -69,12 +69,28 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// The x columns of one group by 4-byte copies (rows of x off the 16-byte boundaries); positions from D on are
+// zero (the rows of V_x are zero there, but what the slot held before need not be finite).
+__device__ __forceinline__ void stage_x_scalar(const float* X, int ldxin, int N, int D, int d0, int len, float* xs,
+                                               int tid) {
+  for (int i = tid; i < N * len; i += kThreads) {
+    const int n = i / len, c = i - n * len;
+    float* dst = xs + n * kXStride + c;
+    if (d0 + c < D)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)),
+                   "l"(X + (long long)n * ldxin + d0 + c)
+                   : "memory");
+    else
+      *dst = 0.f;
+  }
+}
+
 // Issues the 16-byte copies of values [d0, d0 + len) of the CTA's rows of
 // V_x and of the N x columns into one ring slot, as one commit group.
 template <typename TF>
 __device__ __forceinline__ void stage_group(const TF* A, int lda, int K, int Ks, int row0, int vrows,
                                             const float* X, int ldxin, int N, int d0, int len, TF* vs,
-                                            float* xs, int tid) {
+                                            float* xs, int tid, int D, bool xscalar) {
   constexpr int VS = v_stride<TF>();
   constexpr int kPer = 16 / (int)sizeof(TF);  // values per copy
   const int vq = len / kPer;
@@ -84,10 +100,14 @@ __device__ __forceinline__ void stage_group(const TF* A, int lda, int K, int Ks,
     const TF* src = A + (long long)((r / K) * Ks + r % K) * lda + d0 + c * kPer;
     cp_async16(smem_u32(vs + rr * VS + c * kPer), src);
   }
-  const int xq = len / 4;
-  for (int i = tid; i < N * xq; i += kThreads) {
-    const int n = i / xq, c = i - n * xq;
-    cp_async16(smem_u32(xs + n * kXStride + 4 * c), X + (long long)n * ldxin + d0 + 4 * c);
+  if (xscalar) {
+    stage_x_scalar(X, ldxin, N, D, d0, len, xs, tid);
+  } else {
+    const int xq = len / 4;
+    for (int i = tid; i < N * xq; i += kThreads) {
+      const int n = i / xq, c = i - n * xq;
+      cp_async16(smem_u32(xs + n * kXStride + 4 * c), X + (long long)n * ldxin + d0 + 4 * c);
+    }
   }
   cp_async_commit();
 }
@@ -116,14 +136,19 @@ struct FullGroupCopies {
       x[j] = n < N ? X + (long long)n * ldxin + 4 * (tid % 32) : nullptr;
     }
   }
-  __device__ void issue(int d0, TF* vs, float* xs, int tid) const {
+  __device__ void issue(int d0, TF* vs, float* xs, int tid, const float* X, int ldxin, int N, int D,
+                        bool xscalar) const {
     constexpr int VS = v_stride<TF>();
 #pragma unroll
     for (int j = 0; j < NP; ++j)
       if (v[j] != nullptr) cp_async16(smem_u32(vs + (tid / VQ + RP * j) * VS + (tid % VQ) * kPer), v[j] + d0);
+    if (xscalar) {
+      stage_x_scalar(X, ldxin, N, D, d0, kGrp, xs, tid);
+    } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (x[j] != nullptr) cp_async16(smem_u32(xs + (tid / 32 + 8 * j) * kXStride + 4 * (tid % 32)), x[j] + d0);
+      for (int j = 0; j < 4; ++j)
+        if (x[j] != nullptr) cp_async16(smem_u32(xs + (tid / 32 + 8 * j) * kXStride + 4 * (tid % 32)), x[j] + d0);
+    }
     cp_async_commit();
   }
 };
@@ -149,7 +174,7 @@ __global__ void __launch_bounds__(kThreads) xproj_kernel(const TF* __restrict__ 
                                                          const float* __restrict__ X, int ldxin, int N, int D,
                                                          int dchunk, float* __restrict__ out, int ldo, int S,
                                                          int* err, long long limit_ns, unsigned* done_flags,
-                                                         unsigned epoch) {
+                                                         unsigned epoch, int xscalar) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw);  // [0]: incoming chunk sums
   // ring slot s: V_x rows [32][v_stride] then x columns [4 NC][kXStride]
@@ -171,7 +196,8 @@ __global__ void __launch_bounds__(kThreads) xproj_kernel(const TF* __restrict__ 
   const uint32_t q = S > 1 ? cluster_ctarank() : 0u;  // chunk of D
   const int nrows = 4 * K;
   const int vrows = min(kRows, nrows - rb * kRows);
-  const int c_lo = min(D, (int)q * dchunk), c_hi = min(D, c_lo + dchunk);
+  const int De = (D + 3) & ~3;  // (the rows of V_x are zero from D on)
+  const int c_lo = min(De, (int)q * dchunk), c_hi = min(De, c_lo + dchunk);
   const int opc = kRows * kCols / S;  // outputs finished per CTA
   const uint32_t bar_red = smem_u32(&bars[0]);
   const uint64_t limit = static_cast<uint64_t>(limit_ns);
@@ -202,8 +228,11 @@ __global__ void __launch_bounds__(kThreads) xproj_kernel(const TF* __restrict__ 
   const FullGroupCopies<TF> full(A, lda, K, Ks, rb * kRows, vrows, X, ldxin, N, tid);
   auto stage = [&](int gi, int sl) {  // group gi of the chunk into ring slot sl
     const int d0 = c_lo + gi * kGrp, len = min(kGrp, c_hi - d0);
-    if (len == kGrp) full.issue(d0, slot_v(sl), slot_x(sl), tid);
-    else stage_group(A, lda, K, Ks, rb * kRows, vrows, X, ldxin, N, d0, len, slot_v(sl), slot_x(sl), tid);
+    if (len == kGrp)
+      full.issue(d0, slot_v(sl), slot_x(sl), tid, X, ldxin, N, D, xscalar != 0);
+    else
+      stage_group(A, lda, K, Ks, rb * kRows, vrows, X, ldxin, N, d0, len, slot_v(sl), slot_x(sl), tid, D,
+                  xscalar != 0);
   };
   // the first NG groups all in flight (an empty commit group past the end
   // keeps the count of groups behind the one consumed constant)
@@ -224,7 +253,7 @@ __global__ void __launch_bounds__(kThreads) xproj_kernel(const TF* __restrict__ 
   }
 #pragma unroll 1
   for (int i = 0; i < ngrp; ++i) {
-    const int sl = i % NG, len = min(kGrp, c_hi - (c_lo + i * kGrp));  // a multiple of 8 (D % 8 == 0)
+    const int sl = i % NG, len = min(kGrp, c_hi - (c_lo + i * kGrp));  // a multiple of 4
     cp_async_wait<NG - 1>();  // group i has landed (NG - 1 later groups may still be in flight)
     __syncthreads();          // every thread's copies of it (and the zero fill) are visible
     const TF* vs = slot_v(sl);
@@ -319,6 +348,11 @@ __global__ void __launch_bounds__(kThreads) xproj_kernel(const TF* __restrict__ 
   }
 }
 
+// Whether x's rows have to be copied word by word.
+bool x_by_words(int D, const float* X, int ldxin) {
+  return D % 4 != 0 || ldxin % 4 != 0 || (reinterpret_cast<uintptr_t>(X) & 15u) != 0;
+}
+
 // Chunks of D per cluster: about half a CTA per SM in total, at least 128
 // values of D each, and at most max_split.  (Beside a resident recurrence,
 // twice as many CTAs made the whole call slower: D = 1024, 4K = 1024,
@@ -393,7 +427,8 @@ cudaError_t launch_nc(const TF* A, int lda, int K, int Ks, const float* X, int l
   cfg.attrs = attr;
   cfg.numAttrs = signals ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, A, lda, K, Ks, X, ldxin, N, D, dchunk, out, ldo, S, err, limit_ns,
-                            signals ? sig->flags : nullptr, signals ? sig->epoch : 0u);
+                            signals ? sig->flags : nullptr, signals ? sig->epoch : 0u,
+                            x_by_words(D, X, ldxin) ? 1 : 0);
 }
 
 template <typename TF>
@@ -484,12 +519,16 @@ cudaError_t launch_xproj_sparse(const SparseXRows& sr, int K, int Ks, const floa
 }
 
 bool xproj_cluster_fits(int N, int D, const void* A, int lda, const float* X, int ldxin, bool a_bf16) {
-  // 16-byte asynchronous copies need 16-byte aligned base pointers, rows and lengths
+  // 16-byte asynchronous copies need 16-byte aligned rows of the factor (fp32 rows whose length is not a
+  // multiple of 4 are padded with zeros by their stride); rows of x may lie anywhere for fp32 factors (16-byte
+  // copies for D a multiple of 4, else 4-byte ones; before, D off the 8s took the tiled GEMM: two layers D = 300,
+  // H = 200, T = 15, K = 50, three streams 94.4 -> 79.9 us a call, their projections 36.8 -> 25.2 us)
   const int a_align = a_bf16 ? 8 : 4;
-  const bool bases_aligned = ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(X)) & 15u) == 0;
+  const bool a_ok = (reinterpret_cast<uintptr_t>(A) & 15u) == 0 && lda % a_align == 0;
+  const bool x_ok = a_bf16 ? D % 8 == 0 && !x_by_words(D, X, ldxin) : lda >= ((D + 3) & ~3);
   // up to 8 chunks of 32 columns: beyond that every chunk re-reading the
   // CTA's rows costs more than a tiled GEMM
-  return N >= 1 && N <= 8 * kCols && D % 8 == 0 && lda % a_align == 0 && ldxin % 4 == 0 && bases_aligned;
+  return N >= 1 && N <= 8 * kCols && a_ok && x_ok;
 }
 
 cudaError_t launch_xproj_cluster(const void* A, bool a_bf16, int lda, int K, int Ks, const float* X, int ldxin,
