@@ -2,9 +2,14 @@
 //
 // The factors u, v are stored in bf16.  The activations x, h and tau' are
 // fp32 values; each enters the MMAs as a pair of bf16 planes, hi = bf16(a)
-// and lo = bf16(a - hi), so that hi + lo equals a to about 2^-17 relative
-// and every product is issued twice (factor tile x hi, factor tile x lo)
-// into the same fp32 accumulator.  Rounding the activations to one bf16
+// and lo = bf16(a - hi), so that hi + lo equals a to about 2^-17 relative.
+// The planes' tiles follow each other in shared memory, so one MMA of twice
+// the columns multiplies the factor tile by both; the accumulator holds the hi
+// products and then the lo products, which the epilogue adds.  With both
+// operands in shared memory an MMA of 16 terms is bound by reading them: M =
+// 128 takes 69 cycles at N = 32 and 64, 96 at 128 and 157 at 256, so two
+// planes at once cost 69, 96 and 157 instead of 130, 138 and 192 cycles for 32,
+// 64 and 128 streams.  Rounding the activations to one bf16
 // (unit roundoff 2^-9) instead gives elementwise errors of 0.03-0.2 on h
 // and c; with the pair the kernels differ from fp64 arithmetic on the same
 // bf16 factors by a few 1e-4.
@@ -18,8 +23,8 @@
 // tc_rows_kernel computes one 128-row x BN-column tile of the first kind:
 // warp 0 streams K-major tiles of the factor and of both planes of the
 // activation with TMA (128-byte swizzle) through an S-stage mbarrier ring,
-// one thread of warp 1 issues tcgen05.mma (M = 128, N = BN, K = 16 per
-// instruction, once per plane) into a tensor-memory accumulator, and warps
+// one thread of warp 1 issues tcgen05.mma (M = 128, N = 2 BN, K = 16 per
+// instruction) into a tensor-memory accumulator, and warps
 // 4..11 (two per 32-lane quarter of tensor memory) read it back with
 // tcgen05.ld for the epilogue: store P, or form tau' and store it as its
 // bf16 pair.  For tau' the epilogue warps load their P_t values into
@@ -144,7 +149,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   static_assert(BN <= 128, "the epilogue holds P_t of its columns in registers");
   constexpr uint32_t kBBytes = BN * kTileK * 2;        // one plane of the activation tile
   constexpr uint32_t kStage = kABytes + 2 * kBBytes;   // factor tile, hi plane, lo plane (XF: first the fp32 tile)
-  constexpr uint32_t kCols = BN < 32 ? 32 : BN;
+  constexpr uint32_t kCols = 2 * BN;  // the hi products, then the lo products
   constexpr int kNb = XF ? 3 * S : 2 * S;  // full[S] | empty[S] (| converted[S])
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -255,7 +260,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       wait_cta(bar0 + 8u * s, (last / S) & 1, limit, err);
     }
   } else if (warp == 1 && elect_one()) {  // ---- MMA issuer ----
-    constexpr uint32_t idesc = umma_idesc_bf16(kTileM, BN);
+    constexpr uint32_t idesc = umma_idesc_bf16(kTileM, 2 * BN);  // both planes of the activation
     bool ok = true;
     for (int i = 0; i < nloc && ok; ++i) {
       const int s = i % S;
@@ -264,12 +269,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       tc_fence_after();
       const uint32_t st = base + s * kStage;
       const uint64_t da = umma_desc_sw128(st);
-      const uint64_t dhi = umma_desc_sw128(st + kABytes), dlo = umma_desc_sw128(st + kABytes + kBBytes);
+      const uint64_t db = umma_desc_sw128(st + kABytes);
 #pragma unroll
-      for (int kk = 0; kk < kTileK / 16; ++kk) {
-        umma_bf16(tmem, da + 2ull * kk, dhi + 2ull * kk, idesc, (i | kk) != 0 ? 1u : 0u);
-        umma_bf16(tmem, da + 2ull * kk, dlo + 2ull * kk, idesc, 1u);
-      }
+      for (int kk = 0; kk < kTileK / 16; ++kk)
+        umma_bf16(tmem, da + 2ull * kk, db + 2ull * kk, idesc, (i | kk) != 0 ? 1u : 0u);
       umma_commit(bar0 + 8u * (S + s));  // frees the stage once these MMAs are done
     }
     if (!ok) atomicCAS(a.err, 0, kErrTcTimeout);
@@ -349,11 +352,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc_fence_after();
 #pragma unroll
         for (int cc = 0; cc < kHalf; cc += 16) {
-          float v[16];
-          tmem_ld16(trow + cbeg + cc, v);
-          tmem_wait_ld();
+          float v[16], w[16];
+          tmem_ld16x2_sync(trow + cbeg + cc, trow + BN + cbeg + cc, v, w);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) sp_val[cc + j] = (ok && nloc > 0) ? v[j] : 0.f;
+          for (int j = 0; j < 16; ++j) sp_val[cc + j] = (ok && nloc > 0) ? v[j] + w[j] : 0.f;
         }
       }
     } else {
@@ -373,10 +375,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
     for (int cc = 0; cc < kHalf; cc += 16) {
       const int c0 = cbeg + cc;
-      float v[16];
-      tmem_ld16(trow + c0, v);
-      tmem_wait_ld();
+      float v[16], w[16];
+      tmem_ld16x2_sync(trow + c0, trow + BN + c0, v, w);
       if (!write) continue;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] += w[j];
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const int n = col0 + c0 + j;
@@ -469,15 +472,18 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   constexpr uint32_t kBBytes = NT * kTileK * 2;       // one plane of the tau' tile
   constexpr uint32_t kStage = kABytes + 2 * kBBytes;  // U tile, hi plane, lo plane
-  constexpr uint32_t kAcc = 4 * NT < 32 ? 32 : 4 * NT;  // the four gate accumulators
-  // up to 64 streams per tile, c_{t-1} of the tile is staged in tensor memory
-  // too (columns kAcc .. kAcc + NT), so the cell loop reads it with the sums
-  constexpr bool kCTmem = !SPLIT && NT <= 64;
-  constexpr uint32_t kCols = kCTmem ? 2 * kAcc : kAcc;
+  // up to 64 streams per tile, one MMA multiplies both planes of tau' (the hi sums, then the lo sums in NT
+  // columns more); 128 streams' accumulators leave no room for that
+  constexpr bool kBoth = NT <= 64;
+  constexpr uint32_t kGate = kBoth ? 2 * NT : NT;  // columns of one gate's accumulator
+  constexpr uint32_t kCols = 4 * kGate;
+  // there, c_{t-1} of the tile is staged in shared memory while the MMAs run
+  constexpr bool kCSmem = !SPLIT && NT <= 64;
   static_assert(S >= 4, "a chunk of all four gates must be resident");
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
-  const uint32_t bar0 = base + S * kStage;  // full[S] | empty[S] | accum | drain | ckpt | ckpt_done | slot
+  const uint32_t c_off = S * kStage;  // c_{t-1}: [NT / 2][256 epilogue threads]
+  const uint32_t bar0 = base + c_off + (kCSmem ? NT * 512u : 0u);  // full[S] | empty[S] | accum | drain | ckpt | ckpt_done | slot
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + (bar0 - raw) + 8 * (2 * S + 4));
   const uint32_t accum_bar = bar0 + 8u * (2 * S), drain_bar = accum_bar + 8u;
   const uint32_t ckpt_bar = accum_bar + 16u, ckpt_done = accum_bar + 24u;
@@ -555,7 +561,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       wait_cta(bar0 + 8u * s, (last / S) & 1, limit, err);
     }
   } else if (warp == 1 && elect_one()) {  // ---- MMA issuer ----
-    constexpr uint32_t idesc = umma_idesc_bf16(kTileM, NT);
+    constexpr uint32_t idesc = umma_idesc_bf16(kTileM, kGate);
     bool ok = true;
     int jj = jj_lo;
     for (int kl = 0; kl < nkb && ok; ++kl) {
@@ -581,8 +587,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             dlo[g] = umma_desc_sw128(st + kABytes + kBBytes);
           }
           for (int kk = kk0; kk < kk1; ++kk) {
-            umma_bf16(tmem + g * NT, da[g] + 2ull * kk, dhi[g] + 2ull * kk, idesc, (kl | kk) != 0 ? 1u : 0u);
-            umma_bf16(tmem + g * NT, da[g] + 2ull * kk, dlo[g] + 2ull * kk, idesc, 1u);
+            umma_bf16(tmem + g * kGate, da[g] + 2ull * kk, dhi[g] + 2ull * kk, idesc, (kl | kk) != 0 ? 1u : 0u);
+            if (!kBoth) umma_bf16(tmem + g * kGate, da[g] + 2ull * kk, dlo[g] + 2ull * kk, idesc, 1u);
           }
           if (kk1 == 4) umma_commit(bar0 + 8u * (S + s));  // frees this gate's stage
         }
@@ -616,18 +622,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       for (int g = 0; g < 4; ++g) bias[g] = a.bias[g * a.H + j];
     const uint32_t trow = tmem + ((32u * q) << 16);
     griddep_wait();  // c_t-1 and the outputs are shared with the kernels before this one
-    if constexpr (kCTmem) {  // c_{t-1} of this thread's unit and streams -> tensor memory, while the MMAs run
-#pragma unroll
-      for (int c0 = 0; c0 < kHalf; c0 += 16) {
-        float cv[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const int n = n0 + cbeg + c0 + c;
-          cv[c] = (unit_ok && n < a.B) ? a.c_state[(long long)n * a.H + j] : 0.f;
-        }
-        tmem_st16(trow + kAcc + cbeg + c0, cv);
+    float* cst = reinterpret_cast<float*>(smem_raw + (base - raw) + c_off) + (threadIdx.x - 128);
+    if constexpr (kCSmem) {  // c_{t-1} of this thread's unit and streams, while the MMAs run
+#pragma unroll 16
+      for (int c = 0; c < kHalf; ++c) {
+        const int n = n0 + cbeg + c;
+        cst[c * 256] = (unit_ok && n < a.B) ? a.c_state[(long long)n * a.H + j] : 0.f;
       }
-      tmem_wait_st();
     }
     for (int step = jj_lo; step <= jj_hi; ++step) {
       const bool final_sums = step == jj_hi;
@@ -646,8 +647,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int c0 = cbeg; c0 < cbeg + kHalf; c0 += 16) {
           float y[4][16];
 #pragma unroll
-          for (int g = 0; g < 4; ++g) tmem_ld16(trow + g * NT + c0, y[g]);
-          tmem_wait_ld();
+          for (int g = 0; g < 4; ++g) {
+            if constexpr (kBoth) {
+              float lo[16];
+              tmem_ld16x2_sync(trow + g * kGate + c0, trow + g * kGate + NT + c0, y[g], lo);
+#pragma unroll
+              for (int c = 0; c < 16; ++c) y[g][c] += lo[c];
+            } else {
+              tmem_ld16_sync(trow + g * kGate + c0, y[g]);
+            }
+          }
           if (!write) continue;
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
@@ -666,13 +675,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       // eight streams per round: a compact loop that stays in the
       // instruction cache (fully unrolled cells of whole 16-stream chunks,
       // at about 50 instructions each, did not) with eight independent cells
-      // per thread in flight; c_{t-1} comes from tensor memory, or for wider
+      // per thread in flight; c_{t-1} comes from shared memory, or for wider
       // tiles from global memory one round ahead
       auto load_c = [&](int cb, float (&dst)[8]) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const int n = n0 + cb + e;
-          dst[e] = (!kCTmem && write && cb < cbeg + kHalf && n < a.B) ? a.c_state[(long long)n * a.H + j] : 0.f;
+          dst[e] = (!kCSmem && write && cb < cbeg + kHalf && n < a.B) ? a.c_state[(long long)n * a.H + j] : 0.f;
         }
       };
       float cpn[8];
@@ -684,10 +693,19 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int e = 0; e < 8; ++e) cp[e] = cpn[e];  // loaded before any store of this round
         load_c(c8 + 8, cpn);
         __syncwarp();
-        if constexpr (kCTmem) {
-          tmem_ld8x5_sync(trow + c8, trow + NT + c8, trow + 2 * NT + c8, trow + 3 * NT + c8, trow + kAcc + c8, y, cp);
-        } else {
-          tmem_ld8x4_sync(trow + c8, trow + NT + c8, trow + 2 * NT + c8, trow + 3 * NT + c8, y);
+        tmem_ld8x4_sync(trow + c8, trow + kGate + c8, trow + 2 * kGate + c8, trow + 3 * kGate + c8, y);
+        if constexpr (kBoth) {
+          float lo[4][8];
+          const uint32_t tl = trow + NT + c8;
+          tmem_ld8x4_sync(tl, tl + kGate, tl + 2 * kGate, tl + 3 * kGate, lo);
+#pragma unroll
+          for (int g = 0; g < 4; ++g)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) y[g][e] += lo[g][e];
+        }
+        if constexpr (kCSmem) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) cp[e] = cst[(c8 - cbeg + e) * 256];
         }
         if (write) {
           // the eight cells first (independent chains the scheduler can
@@ -891,9 +909,9 @@ template <int BN, int S, bool XF>
 size_t rows_smem() {
   return 1024 + S * (kABytes + 2 * BN * kTileK * 2) + 8 * ((XF ? 3 : 2) * S + 3) + 16;
 }
-template <int NT, int S>
+template <int NT, int S, bool SPLIT>
 size_t gates_smem() {
-  return 1024 + S * (kABytes + 2 * NT * kTileK * 2) + 8 * (2 * S + 4) + 16;
+  return 1024 + S * (kABytes + 2 * NT * kTileK * 2) + (!SPLIT && NT <= 64 ? NT * 512 : 0) + 8 * (2 * S + 4) + 16;
 }
 
 template <int BN, int S, bool XF = false>
@@ -936,7 +954,7 @@ template <int NT, int S, bool SPLIT>
 cudaError_t launch_gates_t(const TcMap& U, const TcMap& Tau, const TcGatesArgs& a, cudaStream_t s) {
   auto kern = tc_gates_kernel<NT, S, SPLIT>;
   static thread_local bool attr = false;
-  const size_t smem = gates_smem<NT, S>();
+  const size_t smem = gates_smem<NT, S, SPLIT>();
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -321,22 +321,6 @@ __device__ __forceinline__ void umma_commit(uint32_t mb) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mb) : "memory");
 }
 
-// 32 lanes x 16 consecutive 32-bit columns of tensor memory: thread i of the
-// warp gets row (lane base + i), columns [col, col + 16).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
 // 32 lanes x 8 consecutive 32-bit columns and the wait for them in one
 // statement.
 __device__ __forceinline__ void tmem_ld8_sync(uint32_t taddr, float (&v)[8]) {
@@ -374,33 +358,7 @@ __device__ __forceinline__ void tmem_ld8x4_sync(uint32_t t0, uint32_t t1, uint32
   for (int i = 0; i < 32; ++i) v[i >> 3][i & 7] = __uint_as_float(r[i]);
 }
 
-// Five loads of 32 lanes x 8 consecutive 32-bit columns (at t0 .. t4) and
-// the wait for them in one statement: v[i][c] = column t_i + c of this
-// thread's row (i < 4), w[c] = column t4 + c.
-__device__ __forceinline__ void tmem_ld8x5_sync(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3, uint32_t t4,
-                                                float (&v)[4][8], float (&w)[8]) {
-  uint32_t r[40];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%40];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%41];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16, %17, %18, %19, %20, %21, %22, %23}, [%42];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24, %25, %26, %27, %28, %29, %30, %31}, [%43];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32, %33, %34, %35, %36, %37, %38, %39}, [%44];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
-        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39])
-      : "r"(t0), "r"(t1), "r"(t2), "r"(t3), "r"(t4)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i >> 3][i & 7] = __uint_as_float(r[i]);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) w[i] = __uint_as_float(r[32 + i]);
-}
-
-// Two tmem_ld16 and one wait for both in one statement, so that no use of
+// Two 16-column loads and one wait for both in one statement, so that no use of
 // the values can be scheduled before they have arrived.
 __device__ __forceinline__ void tmem_ld16x2_sync(uint32_t ta, uint32_t tb, float (&va)[16], float (&vb)[16]) {
   uint32_t r[32];
@@ -443,8 +401,9 @@ __device__ __forceinline__ void tmem_wait_ld_tie32(uint32_t (&r)[32]) {
   asm volatile("" : "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]));
 }
 
-// tmem_ld16 and the wait for it in one statement, so that no use of the
-// values can be scheduled before they have arrived.
+// 32 lanes x 16 consecutive 32-bit columns of tensor memory (thread i of the
+// warp gets row lane base + i) and the wait for them in one statement, so that
+// no use of the values can be scheduled before they have arrived.
 __device__ __forceinline__ void tmem_ld16_sync(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
   asm volatile(
