@@ -65,11 +65,15 @@ namespace {
 
 using namespace lstm_approx_dev;
 
-constexpr int kTcThreads = 384;  // warps 0..3: TMA, MMA, TMEM, spare; warps 4..11: epilogue
+constexpr int kTcThreads = 384;  // warps 0..3: TMA, MMA, TMEM, spare; the others: epilogue
 constexpr int kTileM = 128;
 constexpr int kTileK = 64;  // bf16 elements in one 128-byte swizzled row
 constexpr uint32_t kABytes = kTileM * kTileK * 2;
 constexpr int kConvGroups = 2;  // groups of epilogue warps converting alternate stages of fp32 activations
+// Epilogue warps of tc_rows_kernel: 8, or 16 where they convert 128-column tiles for two row tiles (8 took 886
+// us at D=2048, T B=65536, K=512 and 244 at K=128; 16 851 and 239)
+constexpr int rows_epilogue_warps(bool xf, int mt) { return xf && mt > 1 ? 16 : 8; }
+constexpr int rows_threads(bool xf, int mt) { return 128 + 32 * rows_epilogue_warps(xf, mt); }
 
 // Named barrier `id` of `count` threads; returns whether any of them passed `pred`.
 __device__ __forceinline__ bool block_or(int id, int count, bool pred) {
@@ -95,6 +99,14 @@ __device__ __forceinline__ bool wait_cta(uint32_t mb, uint32_t parity, uint64_t 
 __device__ __forceinline__ void bf16_pair(float v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
   hi = __float2bfloat16_rn(v);
   lo = __float2bfloat16_rn(v - __bfloat162float(hi));
+}
+
+// The pairs of two values, each plane's two packed in one word (v0 in the low half).
+__device__ __forceinline__ void bf16_pair2(float v0, float v1, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(v0 - __uint_as_float(hi << 16), v1 - __uint_as_float(hi & 0xFFFF0000u));
+  lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
 __device__ __forceinline__ void bf16x8_to_f32(const uint4& w, float* f) {
@@ -142,14 +154,25 @@ __device__ __forceinline__ float remainder_terms(const TcGatesArgs& a, int g, in
 // columns) lands where the pair goes (both planes: the same bytes); the
 // converting threads read all of it into registers, meet at a named
 // barrier, and write the pair over it.
-template <int BN, int S, bool XF>
-__global__ void __launch_bounds__(kTcThreads, 1)
+//
+// MT = 2 (the projection over many columns): two 128-row tiles per CTA share
+// the activation tile.  One tile of 128 rows x 128 columns takes 48 KB per 64
+// terms, and at 107 GB/s into an SM that, not the tensor pipe, bounded it; two
+// take 64 KB for twice the work (D=2048, T B=65536, K=512: 813 -> 722 us, now
+// bound by the MMAs' operand reads, 1256 of about 1560 cycles per 64 terms,
+// and the start and end of each tile).  Converting x inside adds 64 KB of
+// shared-memory traffic per 64 terms to the 160 KB of copies and operand reads:
+// 851 us, against 722 and 165 for the pass before.
+template <int BN, int S, bool XF, int MT>
+__global__ void __launch_bounds__(rows_threads(XF, MT), 1)
     tc_rows_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tmb, TcRowsArgs a) {
   extern __shared__ uint8_t smem_raw[];
   static_assert(BN <= 128, "the epilogue holds P_t of its columns in registers");
   constexpr uint32_t kBBytes = BN * kTileK * 2;        // one plane of the activation tile
-  constexpr uint32_t kStage = kABytes + 2 * kBBytes;   // factor tile, hi plane, lo plane (XF: first the fp32 tile)
-  constexpr uint32_t kCols = 2 * BN;  // the hi products, then the lo products
+  constexpr int kEw = rows_epilogue_warps(XF, MT);
+  constexpr uint32_t kTileA = MT * kABytes;
+  constexpr uint32_t kStage = kTileA + 2 * kBBytes;    // factor tiles, hi plane, lo plane (XF: first the fp32 tile)
+  constexpr uint32_t kCols = MT * 2 * BN;  // per row tile the hi products, then the lo products
   constexpr int kNb = XF ? 3 * S : 2 * S;  // full[S] | empty[S] (| converted[S])
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -159,13 +182,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t conv0 = bar0 + 8u * (2 * S);  // converted[s] (XF)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = blockIdx.x / a.kt_per_gate, kt = blockIdx.x % a.kt_per_gate;
+  const int g = (MT * blockIdx.x) / a.kt_per_gate, kt = (MT * blockIdx.x) % a.kt_per_gate;
   const int row0 = g * a.Ks + kt * kTileM;
+  auto tile_row = [&](int m) {  // first storage row of this CTA's row tile m
+    const int tile = MT * (int)blockIdx.x + m;
+    return tile / a.kt_per_gate * a.Ks + tile % a.kt_per_gate * kTileM;
+  };
   // packed gates (a.rpg > 0, K <= rpg <= 32): the tile's rows are the first
   // rpg terms of each gate, gate g at tile rows [g rpg, (g + 1) rpg), loaded
   // by four copies of rpg rows; tile rows from 4 rpg on stay zero
   const int rpg = a.rpg;
-  const uint32_t a_bytes = rpg > 0 ? 4u * rpg * kTileK * 2 : kABytes;
+  const uint32_t a_bytes = rpg > 0 ? 4u * rpg * kTileK * 2 : kTileA;
   const int col0 = blockIdx.y * BN;
   const int nkb = (a.Kdim + kTileK - 1) / kTileK;
   // reduction axis split over the sk CTAs of a cluster (grid z, mode 1):
@@ -187,7 +214,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     for (int i = 0; i < S; ++i) {
       mbar_init(bar0 + 8u * i, 1);
       mbar_init(bar0 + 8u * (S + i), 1);
-      if (XF) mbar_init(conv0 + 8u * i, 8 / kConvGroups);  // one arrival per warp of the stage's converting group
+      if (XF) mbar_init(conv0 + 8u * i, kEw / kConvGroups);  // one arrival per warp of the stage's converting group
     }
     mbar_init(accum_bar, 1);
     mbar_init(drain_bar, 1);
@@ -215,7 +242,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   // the factor copies of one stage into the tile at st
   auto load_a = [&](uint32_t st, uint32_t bar, int kb) {
     if (rpg == 0) {
-      tma_load_2d(st, &tma, bar, kb * kTileK, row0);
+#pragma unroll
+      for (int m = 0; m < MT; ++m) tma_load_2d(st + m * kABytes, &tma, bar, kb * kTileK, m == 0 ? row0 : tile_row(m));
     } else {
 #pragma unroll
       for (int gg = 0; gg < 4; ++gg) tma_load_2d(st + gg * rpg * kTileK * 2, &tma, bar, kb * kTileK, gg * a.Ks);
@@ -245,11 +273,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         load_a(st, bar0 + 8u * s, kb);
       }
       if constexpr (XF) {  // the fp32 tile, columns [64 kb, 64 kb + 32) and [64 kb + 32, 64 kb + 64)
-        tma_load_2d(st + kABytes, &tmb, bar0 + 8u * s, kb * kTileK, col0);
-        tma_load_2d(st + kABytes + BN * 128u, &tmb, bar0 + 8u * s, kb * kTileK + 32, col0);
+        tma_load_2d(st + kTileA, &tmb, bar0 + 8u * s, kb * kTileK, col0);
+        tma_load_2d(st + kTileA + BN * 128u, &tmb, bar0 + 8u * s, kb * kTileK + 32, col0);
       } else {
-        tma_load_2d(st + kABytes, &tmb, bar0 + 8u * s, kb * kTileK, col0);                      // hi plane
-        tma_load_2d(st + kABytes + kBBytes, &tmb, bar0 + 8u * s, kb * kTileK, a.b_plane + col0);  // lo plane
+        tma_load_2d(st + kTileA, &tmb, bar0 + 8u * s, kb * kTileK, col0);                      // hi plane
+        tma_load_2d(st + kTileA + kBBytes, &tmb, bar0 + 8u * s, kb * kTileK, a.b_plane + col0);  // lo plane
       }
       ++issued;
     }
@@ -269,10 +297,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       tc_fence_after();
       const uint32_t st = base + s * kStage;
       const uint64_t da = umma_desc_sw128(st);
-      const uint64_t db = umma_desc_sw128(st + kABytes);
+      const uint64_t db = umma_desc_sw128(st + kTileA);
 #pragma unroll
       for (int kk = 0; kk < kTileK / 16; ++kk)
-        umma_bf16(tmem, da + 2ull * kk, db + 2ull * kk, idesc, (i | kk) != 0 ? 1u : 0u);
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+          umma_bf16(tmem + m * 2 * BN, da + (uint64_t)(m * (kABytes >> 4)) + 2ull * kk, db + 2ull * kk, idesc,
+                    (i | kk) != 0 ? 1u : 0u);
       umma_commit(bar0 + 8u * (S + s));  // frees the stage once these MMAs are done
     }
     if (!ok) atomicCAS(a.err, 0, kErrTcTimeout);
@@ -281,26 +312,31 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     wait_cta(drain_bar, 0, limit, err);
   } else if (warp >= 4) {  // ---- epilogue: warps 4..11, two per lane quarter ----
     const int ep = warp - 4, q = ep & 3;
-    constexpr int kHalf = BN / 2;
+    constexpr int kHalf = BN / (kEw / 4);  // columns per epilogue warp
     if constexpr (XF) {  // each stage's fp32 activation tile -> its bf16 pair, in place
       // kConvGroups groups of warps take the stages in turn (group g: stages kb = g mod kConvGroups),
       // so that several stages are converted at once
-      constexpr int kGt = 256 / kConvGroups;  // threads per group
+      constexpr int kGt = 32 * kEw / kConvGroups;  // threads per group
       static_assert(BN * 16 % kGt == 0, "whole chunks per thread");
       constexpr int kChunks = BN * 16 / kGt;  // 16-byte chunks of four columns per thread
-      const int grp = ep / (8 / kConvGroups), ce = (threadIdx.x - 128) % kGt;
+      const int grp = ep / (kEw / kConvGroups), ce = (threadIdx.x - 128) % kGt;
       uint8_t* gbase = smem_raw + (base - raw);
       bool cok = true;
       for (int kb = grp; kb < nkb; kb += kConvGroups) {
         const int s = kb % S;
         // every thread of the group takes the same decision (reduction barrier), so that
         // none of them waits at the group's second barrier for one that left
-        const bool failed = !wait_cta(bar0 + 8u * s, (kb / S) & 1, limit, err);
+        bool failed = false;
+        // Where the groups do not divide the ring, the stage's last use was another group's, and its copy may still
+        // be in flight (copies end in any order): the parity of this use would then read as passed.  That use's
+        // MMAs are waited for first (the use before it was this group's and is over: the MMAs run in order).
+        if (S % kConvGroups != 0 && kb >= S) failed = !wait_cta(bar0 + 8u * (S + s), (kb / S - 1) & 1, limit, err);
+        if (!wait_cta(bar0 + 8u * s, (kb / S) & 1, limit, err)) failed = true;
         if (block_or(1 + 2 * grp, kGt, failed)) {
           cok = false;
           break;
         }
-        uint8_t* st = gbase + s * kStage + kABytes;
+        uint8_t* st = gbase + s * kStage + kTileA;
         // chunk c = row n, columns [4 (c mod 16), +4): box (k4 / 32) of the fp32 tile
         float4 v[kChunks];
 #pragma unroll
@@ -312,18 +348,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
         for (int i = 0; i < kChunks; ++i) {
           const int c = ce + kGt * i, n = c >> 4, k4 = (c & 15) * 4;
-          __nv_bfloat16 h[4], l[4];
-          bf16_pair(v[i].x, h[0], l[0]);
-          bf16_pair(v[i].y, h[1], l[1]);
-          bf16_pair(v[i].z, h[2], l[2]);
-          bf16_pair(v[i].w, h[3], l[3]);
+          uint2 h, l;
+          bf16_pair2(v[i].x, v[i].y, h.x, l.x);
+          bf16_pair2(v[i].z, v[i].w, h.y, l.y);
           const uint32_t o = sw128_offset(n, k4) + (uint32_t)(n >> 3) * 1024u;
-          *reinterpret_cast<uint2*>(st + o) =
-              make_uint2((uint32_t)__bfloat16_as_ushort(h[0]) | ((uint32_t)__bfloat16_as_ushort(h[1]) << 16),
-                         (uint32_t)__bfloat16_as_ushort(h[2]) | ((uint32_t)__bfloat16_as_ushort(h[3]) << 16));
-          *reinterpret_cast<uint2*>(st + kBBytes + o) =
-              make_uint2((uint32_t)__bfloat16_as_ushort(l[0]) | ((uint32_t)__bfloat16_as_ushort(l[1]) << 16),
-                         (uint32_t)__bfloat16_as_ushort(l[2]) | ((uint32_t)__bfloat16_as_ushort(l[3]) << 16));
+          *reinterpret_cast<uint2*>(st + o) = h;
+          *reinterpret_cast<uint2*>(st + kBBytes + o) = l;
         }
         fence_proxy_async_shared();
         __syncwarp();
@@ -372,6 +402,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc_fence_after();
     const float sig = (add_p && row_ok) ? a.sigma[row] : 0.f;
     const bool write = ok && *err == 0;
+    if constexpr (MT > 1) {  // the projection: P of each row tile
+#pragma unroll 1
+      for (int i = 0; i < MT * (kHalf / 16); ++i) {
+        const int m = i / (kHalf / 16), c0 = cbeg + 16 * (i % (kHalf / 16));
+        const int srow = tile_row(m) + lrow;
+        const bool ok_row = (MT * (int)blockIdx.x + m) % a.kt_per_gate * kTileM + lrow < a.K;
+        float v[16], w[16];
+        __syncwarp();
+        tmem_ld16x2_sync(trow + m * 2 * BN + c0, trow + m * 2 * BN + BN + c0, v, w);
+        float* p = a.P + (long long)(col0 + c0) * a.ldp + srow;
+        const int nv = a.N - (col0 + c0);
+        if (write && ok_row)
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (j < nv) p[(long long)j * a.ldp] = v[j] + w[j];
+      }
+    } else {
 #pragma unroll
     for (int cc = 0; cc < kHalf; cc += 16) {
       const int c0 = cbeg + cc;
@@ -393,6 +440,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           a.tau[a.tau_plane + (long long)n * a.ldt + row] = lo;
         }
       }
+    }
     }
     }
   }
@@ -834,13 +882,7 @@ __global__ void to_bf16_kernel(const float* __restrict__ x, int N, int D, __nv_b
     }
     uint32_t hw[4], lw[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      __nv_bfloat16 h0, l0, h1, l1;
-      bf16_pair(v[2 * e], h0, l0);
-      bf16_pair(v[2 * e + 1], h1, l1);
-      hw[e] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-      lw[e] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-    }
+    for (int e = 0; e < 4; ++e) bf16_pair2(v[2 * e], v[2 * e + 1], hw[e], lw[e]);
     reinterpret_cast<uint4*>(out)[i] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
     reinterpret_cast<uint4*>(out)[total + i] = make_uint4(lw[0], lw[1], lw[2], lw[3]);
   }
@@ -900,25 +942,21 @@ cudaError_t launch_pdl_block(Kern kern, dim3 grid, dim3 block, size_t smem, cuda
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
-template <typename Kern, typename... Args>
-cudaError_t launch_pdl(Kern kern, dim3 grid, size_t smem, cudaStream_t s, Args... args) {
-  return launch_pdl_block(kern, grid, dim3(kTcThreads), smem, s, args...);
-}
 
-template <int BN, int S, bool XF>
+template <int BN, int S, bool XF, int MT>
 size_t rows_smem() {
-  return 1024 + S * (kABytes + 2 * BN * kTileK * 2) + 8 * ((XF ? 3 : 2) * S + 3) + 16;
+  return 1024 + S * (MT * kABytes + 2 * BN * kTileK * 2) + 8 * ((XF ? 3 : 2) * S + 3) + 16;
 }
 template <int NT, int S, bool SPLIT>
 size_t gates_smem() {
   return 1024 + S * (kABytes + 2 * NT * kTileK * 2) + (!SPLIT && NT <= 64 ? NT * 512 : 0) + 8 * (2 * S + 4) + 16;
 }
 
-template <int BN, int S, bool XF = false>
+template <int BN, int S, bool XF = false, int MT = 1>
 cudaError_t launch_rows_t(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, int n_cols, cudaStream_t s) {
-  auto kern = tc_rows_kernel<BN, S, XF>;
+  auto kern = tc_rows_kernel<BN, S, XF, MT>;
   static thread_local bool attr = false;
-  const size_t smem = rows_smem<BN, S, XF>();
+  const size_t smem = rows_smem<BN, S, XF, MT>();
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -927,14 +965,15 @@ cudaError_t launch_rows_t(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, 
   static_assert((size_t)kTileM * (BN + 4) * 4 <= (size_t)S * (kABytes + 2 * BN * kTileK * 2),
                 "a split's receive buffer fits over the stage ring");
   const int sk = (!XF && a.sk > 1) ? a.sk : 1;
-  const dim3 grid(a.rpg > 0 ? 1 : 4 * a.kt_per_gate, (n_cols + BN - 1) / BN, sk);
+  const dim3 grid(a.rpg > 0 ? 1 : 4 * a.kt_per_gate / MT, (n_cols + BN - 1) / BN, sk);
   if (sk == 1)
-    return launch_pdl(kern, grid, smem, s, *reinterpret_cast<const CUtensorMap*>(A.bytes),
-                      *reinterpret_cast<const CUtensorMap*>(Bm.bytes), a);
+    return launch_pdl_block(kern, grid, dim3(rows_threads(XF, MT)), smem, s,
+                            *reinterpret_cast<const CUtensorMap*>(A.bytes),
+                            *reinterpret_cast<const CUtensorMap*>(Bm.bytes), a);
   // the sk CTAs of a split tile form one cluster along z
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(kTcThreads);
+  cfg.blockDim = dim3(rows_threads(XF, MT));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attrs[2];
@@ -961,8 +1000,9 @@ cudaError_t launch_gates_t(const TcMap& U, const TcMap& Tau, const TcGatesArgs& 
     attr = true;
   }
   const cudaError_t e =
-      launch_pdl(kern, dim3((a.H + kTileM - 1) / kTileM, (a.B + NT - 1) / NT, a.ks), smem, s,
-                 *reinterpret_cast<const CUtensorMap*>(U.bytes), *reinterpret_cast<const CUtensorMap*>(Tau.bytes), a);
+      launch_pdl_block(kern, dim3((a.H + kTileM - 1) / kTileM, (a.B + NT - 1) / NT, a.ks), dim3(kTcThreads), smem, s,
+                       *reinterpret_cast<const CUtensorMap*>(U.bytes),
+                       *reinterpret_cast<const CUtensorMap*>(Tau.bytes), a);
   if (e != cudaSuccess || !SPLIT) return e;
   const long long total = (long long)a.B * a.H;
   return launch_pdl_block(tc_gates_reduce_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, a);
@@ -1018,7 +1058,8 @@ int tc_gates_tile_n(int H, int B) {
 }
 
 cudaError_t launch_tc_rows_xf32(const TcMap& A, const TcMap& Xf, const TcRowsArgs& a, int n_cols, cudaStream_t s) {
-  return launch_rows_t<64, 6, true>(A, Xf, a, n_cols, s);
+  return a.rpg > 0 ? launch_rows_t<64, 6, true>(A, Xf, a, n_cols, s)
+                   : launch_rows_t<128, 3, true, 2>(A, Xf, a, n_cols, s);
 }
 
 bool tc_make_map_f32(TcMap* m, const void* base, uint64_t inner, uint64_t rows, uint64_t pitch_bytes,
@@ -1055,7 +1096,9 @@ bool tc_make_map_planes(TcMap* m, const void* base, uint64_t inner, uint64_t row
 
 cudaError_t launch_tc_rows(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, int n_cols, int bn, cudaStream_t s) {
   switch (bn) {
-    case 128: return launch_rows_t<128, 4>(A, Bm, a, n_cols, s);
+    case 128:
+      return a.mode == 0 && a.rpg == 0 ? launch_rows_t<128, 3, false, 2>(A, Bm, a, n_cols, s)
+                                       : launch_rows_t<128, 4>(A, Bm, a, n_cols, s);
     case 32: return launch_rows_t<32, 8>(A, Bm, a, n_cols, s);
     default: return launch_rows_t<64, 6>(A, Bm, a, n_cols, s);
   }

@@ -358,11 +358,14 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
   const int pi = rpg == 8 ? 0 : (rpg == 16 ? 1 : 2);
   __nv_bfloat16* in_bf16 = nullptr;
   int ld_in = 0;
-  // packed gates at layer 0: the projection reads x in fp32 and forms its
-  // bf16 pair itself (one tile of rows, so x is converted once either way;
-  // with several row tiles each would convert it again: at K = 512 the
-  // projection took twice as long), where TMA can map x
-  const bool x_f32 = l == 0 && rpg > 0 && D % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
+  // Layer 0's projection reads x in fp32 and forms its bf16 pair itself where TMA can map x, with packed gates
+  // (one tile of rows, x converted once) and over many columns (two row tiles per CTA, each pair of row tiles
+  // converting it again beside its MMAs; the separate pass reads x and writes its pair, the same bytes again).
+  // D=2048, T B=65536, conversion and projection: K=128 402 -> 239 us, K=512 978 -> 851; at K = 1024, D = 4096, T B =
+  // 1024 the pass and the projection from the pair are as fast.
+  const int bnx = tc_rows_tile_n(TB, rpg > 0 ? 1 : 4 * ((K + 127) / 128));
+  const bool x_f32 =
+      l == 0 && (rpg > 0 || (bnx == 128 && K <= 512)) && D % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
   if (l == 0 && !x_f32) {  // operand conversion (outside the timed projection phase)
     LA_CUDA(h, launch_to_bf16(x, TB, D, static_cast<__nv_bfloat16*>(h->x_bf16), s.ldx, h->stream),
             "input conversion launch");
@@ -375,10 +378,8 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
   }
   {
     PhaseTimer pt(h, 0);
-    const int kt = (K + 127) / 128;
-    const int bnx = tc_rows_tile_n(TB, rpg > 0 ? 1 : 4 * kt);
     TcMap mx;
-    const bool mapped = x_f32 ? tc_make_map_f32(&mx, x, D, TB, (uint64_t)D * 4, 64)
+    const bool mapped = x_f32 ? tc_make_map_f32(&mx, x, D, TB, (uint64_t)D * 4, rpg > 0 ? 64 : 128)
                               : tc_make_map(&mx, in_bf16, D, 2ull * TB, (uint64_t)ld_in * 2, bnx);
     if (!mapped) return fail(h, LSTM_APPROX_ECUDA, "tensor map encoding failed for the layer input");
     TcRowsArgs ra{};
@@ -395,7 +396,8 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
     ra.err = h->err;
     ra.limit_ns = limit_ns;
     if (x_f32)
-      LA_CUDA(h, launch_tc_rows_xf32(s.map_vx_p[pi], mx, ra, TB, h->stream), "input projection launch");
+      LA_CUDA(h, launch_tc_rows_xf32(rpg > 0 ? s.map_vx_p[pi] : s.map_vx, mx, ra, TB, h->stream),
+              "input projection launch");
     else
       LA_CUDA(h, launch_tc_rows(rpg > 0 ? s.map_vx_p[pi] : s.map_vx, mx, ra, TB, bnx, h->stream),
               "input projection launch");
