@@ -406,6 +406,8 @@ cudaError_t launch_tc_seq(const TcMap& Vh_p, const TcMap& U64, const TcSeqArgs& 
 
 // All T timesteps of a layer in one launch over all stream tiles, factors
 // resident on chip, h and tau' exchanged through L2 (k_tensor_loop.cu).
+constexpr int kLoopSegTerms = 256;   // terms summed in one accumulator (K > 512)
+constexpr int kLoopMaxCuts = kMaxCheckpoints + 1024 / kLoopSegTerms;
 constexpr int kLoopMaxTiles = 256;   // stream tiles (counters) of one launch
 struct TcLoopPlan {
   int nt;                    // streams per tile
@@ -424,7 +426,11 @@ struct TcLoopPlan {
   uint32_t rxa_bytes, rxb_bytes;
   int stages;                // ring stages of 64 elements x nt streams x 2 planes
   uint32_t smem;
-  int ncut;                  // intermediate depths below K
+  int ndep;                  // intermediate depths below K
+  int ncut;                  // accumulator segments of the terms, less one: they end at cut_k[0 .. ncut) and at K
+  int cut_k[kLoopMaxCuts];
+  int stream_segs;           // 1: the segments take the accumulator regions in turn (no intermediate depths)
+  int dep_segs[kMaxCheckpoints];  // segments that depth i sums
 };
 struct TcLoopArgs : TcLoopPlan {
   int H, K, Ks, B, T;
@@ -449,7 +455,6 @@ struct TcLoopArgs : TcLoopPlan {
   __nv_bfloat16* seq_bf16;   // pair of h_t for the next layer: (t*B + n)*ldh + unit, lo plane at + seq_plane; or null
   long long seq_plane;
   int ck_n;
-  int cut_k[kMaxCheckpoints];
   float* ckpt_h;             // element (j, t, n, unit) at j*ck_stride + (t*B + n)*H + unit, or null
   float* ckpt_c;
   long long ck_stride;

@@ -34,7 +34,9 @@
 // start a new accumulator segment (a depth inside a 16-term slice splits the
 // slice into pieces whose other terms are zero), so no term is multiplied
 // twice: the full depth is the sum of all segments and is finished first; the
-// depths' cells run while the next step's tau' is on its way.
+// depths' cells run while the next step's tau' is on its way.  Long sums
+// (K > 512) are cut into segments as well; without depths these take two
+// accumulators in turn and are added up as they come.
 //
 // What bounds a step is latency and the epilogue's instructions, not bytes or
 // the tensor pipe.  At H = 512, B = 256, K = 512 (SM cycles, CTA 0; 19,500 a
@@ -237,7 +239,9 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
   const int nb = max(0, min(a.sb, a.ST - tb0));
   const int nkh = min(a.nka, (H + 63) / 64 - za * a.nka);  // this CTA's 64-column chunks of H
   const int nkb = (K + 63) / 64, nsl = (K + 15) / 16;
-  const int ncut = a.ncut;
+  const int ncut = a.ncut, ndep = a.ndep;
+  const bool stream = GP == 1 && a.stream_segs != 0;
+  const int reg_segs = stream ? 1 : ncut + 1;  // segments of an accumulator region of role B
   const int regs_a = a.ra_regions, regs_b = a.rb_regions;
   const unsigned h_step = (unsigned)(a.UT * GB), tau_step = (unsigned)(a.RT * ga);  // counts per step and tile
 
@@ -397,7 +401,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
         for (int s = 0; s < nb && ok; ++s) {
           if (!(ok = drained(drain_b, pb, used_b, regs_b))) break;
           tc_fence_after();
-          uint32_t d0 = tmem + a.acc_b + (uint32_t)pb.slot * (ncut + 1) * seg;  // the current segment's accumulators
+          uint32_t d0 = tmem + a.acc_b + (uint32_t)pb.slot * reg_segs * seg;  // the current segment's accumulators
           int cut = 0;
           int next_cut = ncut > 0 ? a.cut_k[0] : INT_MAX;
           uint32_t u_col = tmem;  // the next resident slice (or piece of one), in the order of issue
@@ -422,7 +426,15 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
               u_col += 8 * GP;
             };
             auto next_segment = [&]() {  // the sums up to depth k_j are complete
-              d0 += seg;
+              if (stream) {
+                umma_commit(acc_b + 8u * pb.slot);
+                pb.next(regs_b);
+                ok = drained(drain_b, pb, used_b, regs_b);
+                tc_fence_after();
+                d0 = tmem + a.acc_b + (uint32_t)pb.slot * seg;
+              } else {
+                d0 += seg;
+              }
               acc = 0;
               ++cut;
               next_cut = cut < ncut ? a.cut_k[cut] : INT_MAX;
@@ -586,7 +598,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
     constexpr uint32_t dg = NT * (MB ? 2 : 1), seg = GP * dg;  // columns of a gate's accumulator, of a depth segment
     // c_{t-1} of this thread's cells: with one stream tile and no intermediate depths in registers across
     // the steps, otherwise in memory, by the parity of t (the depths of step t - 1 run during step t)
-    const bool keep_c = nb <= 1 && ncut == 0;
+    const bool keep_c = nb <= 1 && ndep == 0;
     float cp[CPT];
     auto load_c = [&](int t, int n0) {
       const float* src = t == 0 ? a.c0 : (t & 1) ? a.c_state1 : a.c_state;
@@ -632,7 +644,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
     // per unit tile (GP < 4) each sends its gates' sums to the owners of the streams and takes what they
     // sent; `last`: the accumulators are not read again
     auto gate_sums = [&](int region, int nseg, bool last, float (&y)[4][CPT]) -> bool {
-      const uint32_t tc0 = trow + a.acc_b + (uint32_t)region * (ncut + 1) * seg + part * CW;
+      const uint32_t tc0 = trow + a.acc_b + (uint32_t)region * reg_segs * seg + part * CW;
       __syncwarp();
       if constexpr (GP == 4) {
         if (!MB && nseg == 1) {
@@ -652,12 +664,29 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
         const uint32_t buf =
             (setb ? L.rxb : L.rxa) + (u & 1u) * (a.share_rx ? max(a.rxa_bytes, a.rxb_bytes) : a.rxb_bytes);
         if (e == 0) mbar_arrive_expect_tx(rxb, (uint32_t)(4 * 128 * SO * 4));
+        bool got = true;
 #pragma unroll
         for (int g = 0; g < GP; ++g)
 #pragma unroll
           for (int c8 = 0; c8 < CW; c8 += 8) {
             float v[8];
-            load_sums(tc0 + g * dg + c8, nseg, v);
+            if (!stream) {
+              load_sums(tc0 + g * dg + c8, nseg, v);
+            } else {  // (one group of streams, one gate) every segment in its own region
+              load_sums(tc0, 1, v);
+#pragma unroll 1
+              for (int i = 1; i < nseg && got; ++i) {
+                tc_fence_before();
+                warp_arrive(drain_b + 8u * pb.slot);
+                pb.next(regs_b);
+                got = __all_sync(0xffffffffu, mbar_wait_bounded<false>(acc_b + 8u * pb.slot, pb.parity, limit, err));
+                tc_fence_after();
+                float w[8];
+                load_sums(trow + a.acc_b + (uint32_t)pb.slot * seg + part * CW, 1, w);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) v[c] += w[c];
+              }
+            }
 #pragma unroll
             for (int h4 = 0; h4 < 2; ++h4) {
               const int col = part * CW + c8 + 4 * h4, d = col / SO, sp = col - d * SO;
@@ -668,9 +697,9 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           }
         if (last) {
           tc_fence_before();
-          warp_arrive(drain_b + 8u * region);
+          warp_arrive(drain_b + 8u * (stream ? pb.slot : region));
         }
-        const bool got = __all_sync(0xffffffffu, mbar_wait_bounded<true>(rxb, (u >> 1) & 1u, limit, err));
+        got = __all_sync(0xffffffffu, mbar_wait_bounded<true>(rxb, (u >> 1) & 1u, limit, err)) && got;
         const float* rb = reinterpret_cast<const float*>(gb_ + buf) + part * CPT;
 #pragma unroll
         for (int g = 0; g < 4; ++g)
@@ -692,7 +721,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
 #pragma unroll 1
       for (int set = set0; set < set1 && !fail; ++set) {
         float y[4][CPT], hv[CPT], cv[CPT];
-        fail = !gate_sums(region, set == 0 ? ncut + 1 : set, set == ncut, y);
+        fail = !gate_sums(region, set == 0 ? ncut + 1 : a.dep_segs[set - 1], set == ndep, y);
         if (fail) {
           if (set == 0) publish(true, a.h_count, true);  // the barrier where the block's other warps wait
           break;
@@ -708,7 +737,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
         for (int c = 0; c < CPT; c += 2) store_h2(a.h_bf16, a.ldh, a.h_plane, n0 + c, hv[c], hv[c + 1]);
         if (!publish(false, a.h_count + 32 * (tb0 + s), false)) return false;
         // then what nothing waits for
-        for (int jj = ncut; jj < a.ck_n; ++jj) store_depth(jj, t, n0, hv, cv);  // depths of at least K
+        for (int jj = ndep; jj < a.ck_n; ++jj) store_depth(jj, t, n0, hv, cv);  // depths of at least K
         if (a.seq_bf16) {
           __nv_bfloat16* sq = a.seq_bf16 + (long long)t * B * a.ldh;
 #pragma unroll
@@ -745,12 +774,12 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
 #pragma unroll 1
       for (int s = 0; s < nb && !fail; ++s) {
         load_c(t, first_stream(s));
-        fail = !run_sets(t, s, region, 1, ncut + 1);
+        fail = !run_sets(t, s, region, 1, ndep + 1);
         if (++region == regs_b) region = 0;
       }
       return !block_or_named(1, EPI, fail);
     };
-    const bool defer = a.defer_depths != 0 && ncut > 0 && nb > 0;
+    const bool defer = a.defer_depths != 0 && ndep > 0 && nb > 0;
     bool ok = true;
     // h_{-1} = h0 (or zero) of this CTA's units and streams
     for (int s = 0; s < nb && ok; ++s) {
@@ -864,8 +893,8 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
         bool good = got && run_sets(t, s, pb.slot, 0, 1);
         if (!got) good = publish(true, a.h_count, true);
         ok = good;
-        if (ok && ncut > 0 && !defer) {
-          bool fail = !run_sets(t, s, pb.slot, 1, ncut + 1);
+        if (ok && ndep > 0 && !defer) {
+          bool fail = !run_sets(t, s, pb.slot, 1, ndep + 1);
           ok = !block_or_named(1, EPI, fail);
         }
         pb.next(regs_b);
@@ -982,14 +1011,36 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
   p.share_rx = (p.ga == gb || p.ga == 1 || gb == 1) ? 1 : 0;
   // intermediate depths below K; those inside a 16-term slice split it into one more piece
   int pieces = 0, last_split = -1;
-  while (p.ncut < ck.n && ck.k[p.ncut] < K) {
-    if (ck.k[p.ncut] % 16 != 0) {
+  while (p.ndep < ck.n && ck.k[p.ndep] < K) {
+    if (ck.k[p.ndep] % 16 != 0) {
       ++pieces;
-      last_split = ck.k[p.ncut] / 16;
+      last_split = ck.k[p.ndep] / 16;
     }
-    ++p.ncut;
+    ++p.ndep;
   }
+  // The segments: up to each depth, and for K > 512 no longer than kLoopSegTerms, because the rounding of a
+  // long running sum adds up.  Error of h against 64 bits, one accumulator / segments / the two launches (which
+  // split K over CTAs): H = 512, B = 16, K = 902 4.5e-6 / 3.3e-6 / 3.4e-6; H = 256, B = 64, K = 1000
+  // 5.0e-6 / 4.3e-6 / 4.3e-6; at K = 512 one accumulator 3.35e-6, the two launches 3.40e-6.
+  for (int i = 0, at = 0; i <= p.ndep; ++i) {
+    const int end = i < p.ndep ? ck.k[i] : K;
+    if (K > 512)
+      for (int n = (end - at + kLoopSegTerms - 1) / kLoopSegTerms; n > 1; --n)  // n parts of whole slices
+        p.cut_k[p.ncut++] = at = (at + (end - at + n - 1) / n + 8) / 16 * 16;
+    if (i == p.ndep) break;
+    p.cut_k[p.ncut++] = at = end;
+    p.dep_segs[i] = p.ncut;
+  }
+  // without depths to read later, the epilogue adds up the segments as they come, and two accumulators do (H = 2048,
+  // B = 64, K = 1024: four left room for tiles of 16 streams only, 18.4 us a step; two 15.3)
+  p.stream_segs = p.ncut > 0 && p.ndep == 0;
   const int most = p.cs == 4 ? 144 : 148;  // CTAs in one wave: 36 clusters of 4, 74 of 2
+  auto per_cta = [&](int nt, int groups) {  // stream tiles per CTA so that all groups' CTAs fit in one wave (0: none)
+    const int ST = (B + nt - 1) / nt;
+    for (int n = 1; n <= 8; ++n)
+      if ((long long)groups * ((ST + n - 1) / n) <= most) return n;
+    return 0;
+  };
   // fills in the tile width nt with ures 64-term chunks of U in tensor memory; false if it does not fit
   auto fit = [&](int nt, int ures, TcLoopPlan* o) {
     TcLoopPlan c = p;
@@ -997,19 +1048,14 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     c.ures = ures;
     c.ST = (B + nt - 1) / nt;
     if (c.ST > kLoopMaxTiles) return false;
-    auto per_cta = [&](int groups) {  // stream tiles per CTA so that all groups' CTAs fit in one wave
-      for (int n = 1; n <= 8; ++n)
-        if ((long long)groups * ((c.ST + n - 1) / n) <= most) return n;
-      return 0;
-    };
-    c.sa = per_cta(c.RT * c.ga);
-    c.sb = per_cta(c.UT * gb);
+    c.sa = per_cta(nt, c.RT * c.ga);
+    c.sb = per_cta(nt, c.UT * gb);
     // A CTA's epilogues take longer than the launches they save once its stream tiles are many.  Measured
     // (recurrence us a step, this launch / two launches): 96 streams of both roles together (two layers of
     // H = 2048, B = 64, K = 1024 with depths) 24.7 / 35.5; 128 (H = 1024, B = 1024, K = 128) 13.6 / 16.2; 192
-    // (H = 2048, B = 256, K = 200) 16.9 / 20.4, (H = 1024, B = 256, K = 1000) 29.1 / 30.1; 256 (H = 1024,
-    // B = 600, K = 200) 24.0 / 19.1; 384 (H = 2048, B = 256, K = 1000) 36.0 / 34.7.
-    if (c.sa == 0 || c.sb == 0 || (c.sa + c.sb) * nt > 192) return false;
+    // (H = 2048, B = 256, K = 200) 16.9 / 20.4; 256 (H = 1024, B = 600, K = 200) 24.0 / 19.1.  With several
+    // segments of terms 160 (H = 1024, B = 256, K = 640) 18.1 / 23.4; 192 (K = 1000) 33.9 / 25.8.
+    if (c.sa == 0 || c.sb == 0 || (c.sa + c.sb) * nt > (K > 512 ? 160 : 192)) return false;
     c.nA = c.RT * c.ga * ((c.ST + c.sa - 1) / c.sa);
     c.nB = c.UT * gb * ((c.ST + c.sb - 1) / c.sb);
     const int n = c.nA > c.nB ? c.nA : c.nB;
@@ -1020,7 +1066,7 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     if (last_split >= slices) return false;  // pieces of a slice are in tensor memory
     c.ux_chunks = c.gp * (nkb - ures);
     c.acc_a = ((slices + pieces) * c.gp * 8 + 31) / 32 * 32;
-    const int seg = (c.ncut + 1) * c.gp * nt;  // role B's accumulators of one item, one plane's columns
+    const int seg = (c.stream_segs ? 1 : c.ncut + 1) * c.gp * nt;  // role B's accumulators of one region, one plane's columns
     int room = 512 - c.acc_a;
     if (room < seg || room < 2 * nt) return false;
     c.shared_acc = room < seg + 2 * nt ? 1 : 0;
@@ -1029,13 +1075,13 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     // Regions: a second one lets the next item's MMAs run while the epilogue reads this one's sums (with
     // intermediate depths it reads them late), and comes before both planes in one MMA (half the MMAs, but
     // twice the columns).
-    const int want = c.sb > 1 || c.ncut > 0 ? 2 : 1;
+    const int want = c.sb > 1 || c.ndep > 0 || c.stream_segs ? 2 : 1;
     c.mb = room >= 2 * seg * want ? 1 : 0;
     c.rb_regions = room / (seg * (1 + c.mb));
     if (c.rb_regions > kMaxRegions) c.rb_regions = kMaxRegions;
     if (c.rb_regions > want && c.rb_regions > c.sb) c.rb_regions = want > c.sb ? want : c.sb;
     // the intermediate depths wait for the next step's tau' where their accumulators can stay that long
-    c.defer_depths = (c.ncut > 0 && !c.shared_acc && c.rb_regions >= c.sb) ? 1 : 0;
+    c.defer_depths = (c.ndep > 0 && !c.shared_acc && c.rb_regions >= c.sb) ? 1 : 0;
     c.ra_regions = 1;
     if (c.shared_acc) {
       c.ra_regions = room / (2 * nt) < 2 ? room / (2 * nt) : 2;
@@ -1056,10 +1102,20 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     *o = c;
     return true;
   };
-  // Wider tiles issue fewer MMAs and copies.  Among the ways to hold U: separate accumulators for the two
-  // roles first, then as much of U as possible in tensor memory.
+  // Tiles of 16 streams spread a few streams over more CTAs and have half the sums to read and exchange per
+  // item; with many tiles per CTA those of 32 pay each item's latencies less often.  Recurrence, us a step, tiles
+  // of 16 / 32 by the stream tiles of 16 per CTA (both roles; one gate per CTA, no depths unless said): 2 (H = 512,
+  // B = 64, K = 512) 7.5 / 8.7, (K = 128, all gates) 8.0 / 9.0, (K = 512, two depths, B = 128) 9.2 / 10.9; 3 (H =
+  // 512, B = 128, K = 902) 11.6 / 13.3, (H = 1024, B = 64, K = 700, a depth) 12.3 / 13.1; 4 (H = 2048, B = 64,
+  // K = 512) 9.5 / 10.5, (H = 512, B = 1024, K = 128, all gates) 9.9 / 9.2, (H = 512, B = 256, K = 512, two depths)
+  // 12.1 / 11.4; 5 (H = 512, B = 300, K = 200) 10.9 / 10.0; 8 (H = 512, B = 512, K = 512) 15.0 / 11.4.
+  // Among the ways to hold U: separate accumulators for the two roles first, then as much of U as possible in
+  // tensor memory.
   TcLoopPlan c;
-  for (int nt : {32, 16})
+  const int few = p.gp == 1 && p.ndep == 0 ? 4 : 3;
+  const int sa16 = per_cta(16, p.RT * p.ga), sb16 = per_cta(16, p.UT * gb);
+  const int first = sa16 > 0 && sb16 > 0 && sa16 + sb16 <= few ? 16 : 32;
+  for (int nt : {first, 48 - first})
     for (int shared = 0; shared < 2; ++shared)
       for (int ures = nkb; ures >= 0; --ures)
         if (fit(nt, ures, &c) && c.shared_acc == shared) {

@@ -480,7 +480,6 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
     qa.seq_bf16 = top ? nullptr : static_cast<__nv_bfloat16*>(h->seq_bf16);
     qa.seq_plane = (long long)TB * h->ldh;
     qa.ck_n = ck.n;
-    for (int j = 0; j < ck.n; ++j) qa.cut_k[j] = ck.k[j];
     qa.ckpt_h = ckpt_h;
     qa.ckpt_c = ckpt_c;
     qa.ck_stride = (long long)T * B * H;

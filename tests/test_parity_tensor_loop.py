@@ -39,6 +39,9 @@ def _gates(H, C, K, nz, seed):
     (1024, 2, 40, 512, [32, 511]),          # both exchanges, groups of two and four
     (2048, 2, 64, 1024, [16, 64, 256, 1024]),  # terms of U in shared memory, several tiles per CTA
     (256, 2, 300, 1000, []),                # many row tiles: several stream tiles per CTA
+    (512, 3, 40, 513, []),                  # the shortest sum cut into segments
+    (512, 3, 40, 902, [9, 451]),            # depths among the segments, one inside a slice
+    (512, 3, 40, 800, [640]),               # a segment after the last depth
 ])
 def test_small_shapes(cuda_device, H, T, B, K, cps):
     D = 48
@@ -145,6 +148,7 @@ def test_bounded_wait_reports_timeout(cuda_device, H, K):
     (600, 100, 32, [10], 1), (2048, 64, 1024, [16, 256], 1),
     (2049, 16, 64, [], 0), (2048, 16, 1025, [], 0),             # outside its limits
     (1024, 1024, 128, [], 1), (1024, 1024, 512, [], 0),         # too many streams per CTA
+    (1024, 256, 640, [], 1), (1024, 256, 1000, [], 0),
 ])
 def test_rule(H, B, K, cps, loop):
     p = plan(BF16, H, 2, B, K, cps)
