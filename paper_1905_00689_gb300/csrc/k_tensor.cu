@@ -759,10 +759,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           // the eight cells first (independent chains the scheduler can
           // interleave), then their stores
           float hv[8], cv[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            lstm_cell_s(y[0][e] + bias[0], y[1][e] + bias[1], y[2][e] + bias[2], y[3][e] + bias[3], cp[e], hv[e],
-                        cv[e]);
+          lstm_cells_s(y, bias, cp, hv, cv);
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const int n = n0 + c8 + e;

@@ -726,9 +726,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           if (set == 0) publish(true, a.h_count, true);  // the barrier where the block's other warps wait
           break;
         }
-#pragma unroll
-        for (int c = 0; c < CPT; ++c)
-          lstm_cell_s(y[0][c] + bias[0], y[1][c] + bias[1], y[2][c] + bias[2], y[3][c] + bias[3], cp[c], hv[c], cv[c]);
+        lstm_cells_s(y, bias, cp, hv, cv);
         if (set > 0) {
           store_depth(set - 1, t, n0, hv, cv);
           continue;

@@ -219,9 +219,23 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
+// 2^z from the hardware approximation, results below 2^-126 as zero.
+__device__ __forceinline__ float ex2_approx(float z) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(z));
+  return r;
+}
+
+constexpr float kLog2E = 1.44269504088896341f;
+
+// e^z = 2^(z log2 e) for the functions below, all of which add it to 1: a
+// result below 2^-126 may be zero, which saves the scaling around the
+// hardware instruction (three instructions of five).
+__device__ __forceinline__ float exp_for_sum(float z) { return ex2_approx(z * kLog2E); }
+
 // Logistic function 1 / (1 + e^-z) from the hardware exponential and
 // reciprocal: absolute error of a few 1e-7 over the whole range.
-__device__ __forceinline__ float sigmoid_f(float z) { return rcp_approx(1.0f + __expf(-z)); }
+__device__ __forceinline__ float sigmoid_f(float z) { return rcp_approx(1.0f + exp_for_sum(-z)); }
 
 // tanh z with a relative error of a few 1e-7: (1 - e) / (1 + e), e = exp(-2|z|),
 // for |z| >= 1/4, and the Taylor series of tanh to z^9 below (its first
@@ -229,7 +243,7 @@ __device__ __forceinline__ float sigmoid_f(float z) { return rcp_approx(1.0f + _
 // cancellation of 1 - e at small |z|.
 __device__ __forceinline__ float tanh_f(float z) {
   const float a = fabsf(z);
-  const float e = __expf(-2.0f * a);
+  const float e = exp_for_sum(-2.0f * a);
   const float big = copysignf((1.0f - e) * rcp_approx(1.0f + e), z);
   const float z2 = z * z;
   const float poly = z2 * fmaf(z2, fmaf(z2, fmaf(z2, 62.0f / 2835.0f, -17.0f / 315.0f), 2.0f / 15.0f), -1.0f / 3.0f);
@@ -252,14 +266,79 @@ __device__ __forceinline__ float tanh_s(float z) { return fmaf(2.0f, sigmoid_f(2
 // finite; that moves a sigmoid by at most 2.1e-9.
 __device__ __forceinline__ void lstm_cell_s(float yi, float yf, float yg, float yo, float c_prev, float& h_out,
                                             float& c_out) {
-  const float d0 = 1.0f + __expf(-fmaxf(yi, -20.0f)), d1 = 1.0f + __expf(-fmaxf(yf, -20.0f));
-  const float d2 = 1.0f + __expf(-fmaxf(2.0f * yg, -20.0f)), d3 = 1.0f + __expf(-fmaxf(yo, -20.0f));
+  const float d0 = 1.0f + exp_for_sum(-fmaxf(yi, -20.0f)), d1 = 1.0f + exp_for_sum(-fmaxf(yf, -20.0f));
+  const float d2 = 1.0f + exp_for_sum(-fmaxf(2.0f * yg, -20.0f)), d3 = 1.0f + exp_for_sum(-fmaxf(yo, -20.0f));
   const float p01 = d0 * d1, p23 = d2 * d3;
   const float r = rcp_approx(p01 * p23);
   const float r01 = r * p23, r23 = r * p01;  // 1 / (d0 d1), 1 / (d2 d3)
   const float i = r01 * d1, f = r01 * d0, g = fmaf(2.0f, r23 * d3, -1.0f), o = r23 * d2;
   c_out = fmaf(f, c_prev, i * g);
   h_out = o * tanh_s(c_out);
+}
+
+// Two fp32 values in one 64-bit register pair and arithmetic on both at once (one instruction each; the same
+// roundings as the scalar operations).
+__device__ __forceinline__ uint64_t f32x2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f32x2_split(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// lstm_cell_s of N streams (N even) from the gate sums y without bias, two
+// streams per instruction where there is one for two.  The epilogues of the
+// tensor kernels are bound by their instructions: with the plain exponential
+// and one cell at a time a step of H = 1024, B = 1024 took 12.2 us at K = 128
+// (now 11.1) and 23.9 at K = 512 (22.9).
+template <int N>
+__device__ __forceinline__ void lstm_cells_s(const float (&y)[4][N], const float (&bias)[4], const float (&c_prev)[N],
+                                             float (&h_out)[N], float (&c_out)[N]) {
+  const uint64_t one = f32x2(1.0f, 1.0f), two = f32x2(2.0f, 2.0f), neg1 = f32x2(-1.0f, -1.0f);
+  const uint64_t nl = f32x2(-kLog2E, -kLog2E), nl2 = f32x2(-2.0f * kLog2E, -2.0f * kLog2E);
+  auto each = [](uint64_t v, auto f) {
+    float a, b;
+    f32x2_split(v, a, b);
+    return f32x2(f(a), f(b));
+  };
+  auto ex2 = [](float v) { return ex2_approx(v); };
+  auto rcp = [](float v) { return rcp_approx(v); };
+#pragma unroll
+  for (int i = 0; i < N; i += 2) {
+    uint64_t d[4];  // 1 + e^-z of the four gates (z = 2 y for the cell gate)
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const float lim = g == 2 ? -10.0f : -20.0f;
+      const uint64_t z = each(add2(f32x2(y[g][i], y[g][i + 1]), f32x2(bias[g], bias[g])),
+                              [lim](float v) { return fmaxf(v, lim); });
+      d[g] = add2(one, each(mul2(z, g == 2 ? nl2 : nl), ex2));
+    }
+    const uint64_t p01 = mul2(d[0], d[1]), p23 = mul2(d[2], d[3]);
+    const uint64_t r = each(mul2(p01, p23), rcp);
+    const uint64_t r01 = mul2(r, p23), r23 = mul2(r, p01);
+    const uint64_t gi = mul2(r01, d[1]), gf = mul2(r01, d[0]), gg = fma2(two, mul2(r23, d[3]), neg1),
+                   go = mul2(r23, d[2]);
+    const uint64_t c = fma2(gf, f32x2(c_prev[i], c_prev[i + 1]), mul2(gi, gg));
+    const uint64_t th = fma2(two, each(add2(one, each(mul2(c, nl2), ex2)), rcp), neg1);
+    f32x2_split(c, c_out[i], c_out[i + 1]);
+    f32x2_split(mul2(go, th), h_out[i], h_out[i + 1]);
+  }
 }
 
 // Gate nonlinearities and cell update (Sec. II): i, f, o sigmoid, g tanh;
