@@ -141,3 +141,27 @@ def test_seq_kernel_bounded_wait_reports_timeout(cuda_device):
     m.sync()
     ref = oracle_run([gates], x, K, dtype="bf16")
     assert_parity({"h": out.double().cpu().numpy()}, ref, BF16_TOL, keys=("h",))
+
+
+@pytest.mark.parametrize("H,B,K,cps", [
+    (512, 580, 20, [16]),      # the last cluster's second chain has no streams
+    (512, 593, 32, [16, 32]),  # ... has one
+    (1024, 607, 8, []),        # ... has 15; two unit tiles per CTA
+    (1024, 608, 32, [16]),     # whole chains
+    (256, 1170, 17, []),       # clusters of two CTAs
+])
+def test_seq_kernel_two_chains(cuda_device, H, B, K, cps):
+    """More streams than one wave of single chains of 16 holds: two chains per
+    CTA; the last streams and some of either chain."""
+    D, T = 24, 4
+    gates = _gates(H, D + H, K, 40, 7900 + H + K)
+    rng = np.random.default_rng(B)
+    x = draw_inputs(T, B, D, "uniform", 79)
+    h0 = 0.3 * rng.standard_normal((1, B, H))
+    c0 = 0.3 * rng.standard_normal((1, B, H))
+    got, m = run_gpu([gates], x, K, dtype="bf16", h0=h0, c0=c0, checkpoints=cps)
+    assert m.query(Q_TENSOR_SEQ) == 1
+    s = [0, 15, 16, 31, 32, B - 2, B - 1]
+    ref = oracle_run([gates], x[:, s], K, dtype="bf16", h0=h0[:, s], c0=c0[:, s], checkpoints=cps)
+    cut = {k: v[:, s] if k in ("h", "c_last") else v[:, :, s] for k, v in got.items()}
+    assert_parity(cut, ref, BF16_TOL)
