@@ -197,7 +197,7 @@ struct PersistentPlan {
   int RA = 0;        // coefficient rows per CTA (multiple of 4)
   int UB = 0;        // hidden units per CTA (ceil(H / CS) rounded up to 4)
   int upl = 0;       // hidden units per warp (1, 2, 4, 8 or 16; four warps per gate)
-  int kpw = 0;       // refinement terms per lane (1, 2, 4 or 8)
+  int kpw = 0;       // refinement terms per lane (1, 2 or 4)
   int hc = 0;        // 16-value chunks of h per lane in the recurrent product (1 or 2)
   int tcols = 0;     // tensor-memory columns holding the CTA's V_h rows
   size_t smem = 0;   // dynamic shared memory bytes
@@ -254,7 +254,7 @@ cudaError_t launch_persistent_ag(const PersistentAgPlan& plan, const PersistentA
 struct PersistentOnePlan {
   int threads = 0;     // 128, 256 or 512
   int LA = 0, LB = 0;  // lanes per coefficient row, per gate row
-  int VQ = 0;          // quads of either factor per thread (1, 2, 4 or 8)
+  int VQ = 0;          // quads of either factor per thread (1, 2 or 4)
   int HP = 0, KP = 0;  // shared-memory strides of h and of a gate's tau'
 };
 struct OneProj {

@@ -5,7 +5,7 @@
 //
 // The cluster kernels (k_persistent.cu, k_persistent_ag.cu) spend a step on
 // cluster exchanges: about 3000 cycles at H = 64.  Where both factors' h parts
-// fit one CTA's registers (at most 512 threads x 32 values each) there is
+// fit one CTA's registers (at most 512 threads x 16 values each) there is
 // nothing to exchange: a step is two block barriers, two short dot products
 // and the cell, bound by their latency chain (shared-memory reads, FMAs,
 // shuffles, special functions) and by instruction issue.  The fewest threads
@@ -44,7 +44,7 @@ namespace {
 using namespace lstm_approx_dev;
 
 constexpr int kMaxThreads = 512;
-constexpr int kMaxQuads = 8;      // quads of either factor per thread
+constexpr int kMaxQuads = 4;      // quads of either factor per thread
 constexpr int kStepsPerPass = 8;  // timesteps per read of a row's x part
 
 struct OneDev {
@@ -335,22 +335,23 @@ int pow2_at_most(int v) {
 
 bool plan_persistent_one(int H, int K, bool gathers, PersistentOnePlan* out) {
   if (H < 1 || H > 128 || K < 1 || K > 128) return false;
-  // the fewest threads that hold the factors in 4 quads each, else in 8; 512 where compressed rows of x are
-  // gathered (entries in flight)
+  // The fewest threads that hold the factors in 4 quads each; 512 where compressed rows of x are gathered (entries
+  // in flight).  With 8 quads a step takes longer than the one-exchange cluster kernel's and the set-up as long:
+  // T = 32, H = 64, K = 64 55.7 us against 49.7, H = 128, K = 32 57.8 / 45.6, H = 32, K = 96 60.0 / 47.7; with 4
+  // H = 64, K = 32 44.6 / 45.3, H = 32, K = 64 47.5 / 49.7, H = 64, K = 16 33.9 / 43.4.
   PersistentOnePlan p;
-  for (int most : {4, kMaxQuads})
-    for (int nth = 128; nth <= kMaxThreads; nth *= 2) {
-      if (4 * K > nth || 4 * H > nth || (gathers && nth < kMaxThreads)) continue;
-      p.threads = nth;
-      p.LA = pow2_at_most(nth / (4 * K));
-      if (p.LA > 32) p.LA = 32;
-      p.LB = pow2_at_most(nth / (4 * H));
-      if (p.LB > 8) p.LB = 8;
-      const int qa = ((H + 3) / 4 + p.LA - 1) / p.LA, qb = ((K + 3) / 4 + p.LB - 1) / p.LB;
-      const int q = qa > qb ? qa : qb;
-      p.VQ = q <= 1 ? 1 : q <= 2 ? 2 : q <= 4 ? 4 : q <= kMaxQuads ? 8 : 0;
-      if (p.VQ != 0 && p.VQ <= most) goto found;
-    }
+  for (int nth = 128; nth <= kMaxThreads; nth *= 2) {
+    if (4 * K > nth || 4 * H > nth || (gathers && nth < kMaxThreads)) continue;
+    p.threads = nth;
+    p.LA = pow2_at_most(nth / (4 * K));
+    if (p.LA > 32) p.LA = 32;
+    p.LB = pow2_at_most(nth / (4 * H));
+    if (p.LB > 8) p.LB = 8;
+    const int qa = ((H + 3) / 4 + p.LA - 1) / p.LA, qb = ((K + 3) / 4 + p.LB - 1) / p.LB;
+    const int q = qa > qb ? qa : qb;
+    p.VQ = q <= 1 ? 1 : q <= 2 ? 2 : q <= kMaxQuads ? kMaxQuads : 0;
+    if (p.VQ != 0) goto found;
+  }
   return false;
 found:
   p.HP = (H + 3) / 4 * 4;
@@ -369,11 +370,12 @@ size_t persistent_one_smem(const PersistentOnePlan& p, int T, int K, const OnePr
 }
 
 // Whether the projection belongs inside: x of one stream, P and (dense) the rows' x parts in shared memory,
-// and little enough to read for one CTA (64 KB of dense rows, or 32 K kept entries over all timesteps: a
-// separate grid reads more in the time of a launch).
+// and little enough to read for one CTA (64 KB of dense rows, or 28 K kept entries over up to 8 timesteps: a
+// separate grid reads more in the time of a launch: D = 1000, T = 4, K = 32, 25.6 K entries 8.9 us inside, 10.9
+// by its own launch; D = 2000, T = 2, K = 40, 32 K 13.1 / 10.5; D = 500, T = 16, K = 16, 26 K 23.0 / 19.0).
 int persistent_one_projection(int K, int T, int D, long long kept_x, bool sparse) {
   if ((long long)T * D > 16 * 1024 || (long long)T * 4 * K > 12 * 1024) return 0;
-  if (sparse) return kept_x * T <= 32 * 1024 ? 2 : 0;
+  if (sparse) return T <= 8 && kept_x * T <= 28 * 1024 ? 2 : 0;
   return 4LL * K * D <= 16 * 1024 && 4LL * K * (D + 8) <= 20 * 1024 ? 1 : 0;
 }
 
@@ -416,9 +418,9 @@ cudaError_t launch_persistent_one(const PersistentOnePlan& p, const PersistentAr
                                   cudaStream_t s) {
 #define LA_ONE(N_, V_) \
   if (p.threads == N_ && p.VQ == V_) return launch_one_t<N_, V_>(p, a, pr, s);
-  LA_ONE(128, 1) LA_ONE(128, 2) LA_ONE(128, 4) LA_ONE(128, 8)
-  LA_ONE(256, 1) LA_ONE(256, 2) LA_ONE(256, 4) LA_ONE(256, 8)
-  LA_ONE(512, 1) LA_ONE(512, 2) LA_ONE(512, 4) LA_ONE(512, 8)
+  LA_ONE(128, 1) LA_ONE(128, 2) LA_ONE(128, 4)
+  LA_ONE(256, 1) LA_ONE(256, 2) LA_ONE(256, 4)
+  LA_ONE(512, 1) LA_ONE(512, 2) LA_ONE(512, 4)
 #undef LA_ONE
   return cudaErrorInvalidValue;
 }

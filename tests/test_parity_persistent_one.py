@@ -24,8 +24,8 @@ from workloads import draw_factor_set, draw_inputs
     (35, 28, 17, 3, 5, 20, [4], 1, 1),            # D off the 16-byte rows, three passes, several streams
     (8256, 64, 1, 1, 16, 130, [], 1, 1),          # compressed rows inside
     (1000, 64, 3, 2, 4, 20, [2], 1, 1),           # the same, several streams and timesteps
-    (1024, 64, 4, 1, 64, 300, [13], 1, 2),        # 8 quads per thread; projection by its own launch
-    (300, 128, 3, 2, 32, 100, [31], 1, 2),        # the largest H
+    (1024, 64, 4, 1, 32, 300, [13], 1, 2),        # 512 threads; projection by its own launch
+    (300, 128, 3, 2, 16, 100, [15], 1, 2),        # the largest H
     (20, 8, 5, 2, 128, 10, [100, 127], 1, 1),     # the largest K
     (48, 64, 4, 2, 20, 30, [7], 2, 2),            # two layers
     (12, 32, 3, 200, 8, 12, [], 1, 2),            # more streams than SMs: projection by its own launch
@@ -68,9 +68,9 @@ def test_depths_ignore_later_terms_that_are_not_finite(cuda_device):
     assert np.array_equal(np.isfinite(got["h"]), np.isfinite(ref["h"]))
 
 
-@pytest.mark.parametrize("H,K,one", [(64, 16, 1), (64, 64, 1), (64, 65, 0), (128, 32, 1), (128, 33, 0), (129, 4, 0),
-                                     (4, 128, 1), (4, 129, 0), (512, 16, 0)])
+@pytest.mark.parametrize("H,K,one", [(64, 16, 1), (64, 32, 1), (64, 33, 0), (128, 16, 1), (128, 17, 0), (129, 4, 0),
+                                     (32, 64, 1), (32, 65, 0), (4, 128, 1), (4, 129, 0), (512, 16, 0)])
 def test_rule(H, K, one):
-    """H, K <= 128 and at most 32 values of either factor per thread of 512."""
+    """H, K <= 128 and at most 16 values of either factor per thread of 512."""
     if H % 4 == 0:
         assert plan(FP32, H, 4, 1, K)["one_cta"] == one
