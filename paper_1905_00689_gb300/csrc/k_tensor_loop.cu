@@ -1039,6 +1039,15 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
       if ((long long)groups * ((ST + n - 1) / n) <= most) return n;
     return 0;
   };
+  // A CTA's epilogues take longer than the launches they save once its stream tiles are many.  Measured
+  // (recurrence us a step, this launch / two launches): 96 streams of both roles together (two layers of
+  // H = 2048, B = 64, K = 1024 with depths) 21 / 33; 128 (H = 1024, B = 1024, K = 128) 11.1 / 14.6; 192
+  // (H = 2048, B = 256, K = 200) 16.0 / 18.1, (H = 2048, B = 180, K = 512) 16.7 / 18.3, (H = 1024, B = 300, K = 512)
+  // 16.7 / 17.1; 256 (H = 1024, B = 600, K = 200) 22.8 / 15.8.  With several segments of terms 160 (H = 1024,
+  // B = 256, K = 640) 18.1 / 23.4; 192 (K = 1000) 33.9 / 25.8.  Up to K = 320 and H = 1024 without depths the two
+  // launches are at their best: 192 (H = 1024, B = 512, K = 200) 16.7 / 13.6, 160 (H = 512, B = 600, K = 256)
+  // 14.1 / 12.9, 96 (H = 512, B = 400, K = 200) 10.0 / 17.4.
+  const int limit = K > 512 ? 160 : p.gp == 1 && K <= 320 && H <= 1024 && p.ndep == 0 ? 128 : 192;
   // fills in the tile width nt with ures 64-term chunks of U in tensor memory; false if it does not fit
   auto fit = [&](int nt, int ures, TcLoopPlan* o) {
     TcLoopPlan c = p;
@@ -1048,12 +1057,7 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     if (c.ST > kLoopMaxTiles) return false;
     c.sa = per_cta(nt, c.RT * c.ga);
     c.sb = per_cta(nt, c.UT * gb);
-    // A CTA's epilogues take longer than the launches they save once its stream tiles are many.  Measured
-    // (recurrence us a step, this launch / two launches): 96 streams of both roles together (two layers of
-    // H = 2048, B = 64, K = 1024 with depths) 24.7 / 35.5; 128 (H = 1024, B = 1024, K = 128) 13.6 / 16.2; 192
-    // (H = 2048, B = 256, K = 200) 16.9 / 20.4; 256 (H = 1024, B = 600, K = 200) 24.0 / 19.1.  With several
-    // segments of terms 160 (H = 1024, B = 256, K = 640) 18.1 / 23.4; 192 (K = 1000) 33.9 / 25.8.
-    if (c.sa == 0 || c.sb == 0 || (c.sa + c.sb) * nt > (K > 512 ? 160 : 192)) return false;
+    if (c.sa == 0 || c.sb == 0 || (c.sa + c.sb) * nt > limit) return false;
     c.nA = c.RT * c.ga * ((c.ST + c.sa - 1) / c.sa);
     c.nB = c.UT * gb * ((c.ST + c.sb - 1) / c.sb);
     const int n = c.nA > c.nB ? c.nA : c.nB;
@@ -1113,6 +1117,8 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
   const int few = p.gp == 1 && p.ndep == 0 ? 4 : 3;
   const int sa16 = per_cta(16, p.RT * p.ga), sb16 = per_cta(16, p.UT * gb);
   const int first = sa16 > 0 && sb16 > 0 && sa16 + sb16 <= few ? 16 : 32;
+  // (tiles of 16 in place of 32 for want of room do not make more streams fit)
+  if (first == 32 && (per_cta(32, p.RT * p.ga) + per_cta(32, p.UT * gb)) * 32 > limit) return false;
   for (int nt : {first, 48 - first})
     for (int shared = 0; shared < 2; ++shared)
       for (int ures = nkb; ures >= 0; --ures)

@@ -149,6 +149,7 @@ def test_bounded_wait_reports_timeout(cuda_device, H, K):
     (2049, 16, 64, [], 0), (2048, 16, 1025, [], 0),             # outside its limits
     (1024, 1024, 128, [], 1), (1024, 1024, 512, [], 0),         # too many streams per CTA
     (1024, 256, 640, [], 1), (1024, 256, 1000, [], 0),
+    (512, 400, 200, [], 1), (512, 600, 256, [], 0), (512, 600, 256, [100], 1), (2048, 256, 200, [], 1),
 ])
 def test_rule(H, B, K, cps, loop):
     p = plan(BF16, H, 2, B, K, cps)
