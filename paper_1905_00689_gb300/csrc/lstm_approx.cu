@@ -678,6 +678,8 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
     // faster although the projection takes 15.8 instead of 10.5 us).
     // Shorter set-ups gain less than the slower projection costs (K = 64: 4%
     // slower, the one-exchange kernel at K = 16: 11%).
+    // Clusters of 8 start beside a split projection (unsplit / split: D = 1408, H = 124, T = 5, K = 167, 8 streams
+    // 49.6 / 41.4 us, D = 2000, H = 64, T = 4, K = 140, 15 streams 64.0 / 33.3).
     // One stream's factors in one CTA's registers: nothing is exchanged, and a small projection runs inside
     // (D = 64, H = 64, T = 8, K = 16, one stream: 24.2 -> 10.7 us a call; the case-study shape, D = 8256, H = 64, T = 1,
     // K = 16 at 130 kept entries: 8.2 -> 5.8 us).  Forced kernels, clusters and projections take the others.
@@ -719,7 +721,9 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
     const int proj_ctas = rec_first ? xproj_cluster_ctas(K, T * B, s.D, 8) : 0;
     rec_first = rec_first && proj_ctas <= kProjFlags && xproj_cluster_prepare(bf16, T * B) == cudaSuccess;
     const int xproj_max_split =
-        rec_first ? 8 : (path == LSTM_APPROX_PATH_PERSISTENT && !use_one && plan.variant == 1 && K > 128) ? 1 : 8;
+        rec_first ? 8
+        : (path == LSTM_APPROX_PATH_PERSISTENT && !use_one && plan.variant == 1 && plan.CS == 16 && K > 128) ? 1
+                                                                                                          : 8;
     XprojSignal sig;
     if (rec_first) {
       if (++h->proj_epoch == 0) ++h->proj_epoch;  // the flags start at zero
