@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       if (!ok) atomicCAS(a.err, 0, kErrTcTimeout);
       // every issued copy has landed before the CTA may leave
       mbar_wait_bounded<false>(setup_bar, 0, limit, err);
-      for (int s = 0; s < it; ++s)  // slot s was last filled in this round (before the position) or the one before
+      for (int s = 0; s < it; ++s)  // slot s was last filled in this turn of the ring (before the position) or the one before
         mbar_wait_bounded<false>(full0 + 8u * s, s < pos.slot ? pos.parity : pos.parity ^ 1u, limit, err);
     }
   } else if (warp == 1) {

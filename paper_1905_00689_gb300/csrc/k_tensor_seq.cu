@@ -41,7 +41,7 @@
 // What bounds a step (H = 1024, B = 512, K = 8, one chain, 3.6 us, SM cycles):
 // partial tau' 300 after the last h, exchange 1 650, tau' 350, exchange 2 800,
 // gate products 650, cells 900 + 400 (pair, hand-over) per unit tile, stores
-// 500 per unit tile.  The cells are about 70 instructions each, two streams to
+// 500 per unit tile.  The cells are about 75 instructions each, two streams to
 // an instruction where there is one (104 before: 5.1 us a step).  Two chains
 // per CTA (B > 576) let one's exchanges run beside the other's cells: H = 1024,
 // B = 1024, K = 8 / 32 6.7 / 7.9 us a step as one chain of 32, now 5.2 / 5.5;
