@@ -87,6 +87,7 @@ __device__ __forceinline__ bool block_or(int id, int count, bool pred) {
   return r != 0u;
 }
 __device__ __forceinline__ void named_barrier(int id, int count) {
+  __syncwarp();
   asm volatile("barrier.cta.sync.aligned %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 

@@ -145,6 +145,7 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
 // Two loads of 32 lanes x 8 consecutive columns and the wait for both in one statement.
 __device__ __forceinline__ void tmem_ld8x2_sync(uint32_t ta, uint32_t tb, float (&va)[8], float (&vb)[8]) {
   uint32_t r[16];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n\t"
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n\t"
@@ -162,6 +163,7 @@ __device__ __forceinline__ void tmem_ld8x2_sync(uint32_t ta, uint32_t tb, float 
 
 // Store 8 consecutive 32-bit columns per lane into tensor memory; complete with tmem_wait_st().
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8]) {
+  __syncwarp();
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
                "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
                "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),

@@ -154,9 +154,11 @@ struct FullGroupCopies {
 };
 
 __device__ __forceinline__ void cluster_arrive_release() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait_acquire() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

@@ -43,7 +43,12 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
   return r;
 }
 
+// Instructions that end in `.aligned` must be executed by all lanes of a warp
+// together.  A branch that only some lanes take (one lane arming a barrier,
+// lanes leaving a wait at different polls) does not by itself bring them back
+// together, so every wrapper of such an instruction starts with __syncwarp().
 __device__ __forceinline__ void cluster_sync_all() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -371,13 +376,16 @@ __device__ __forceinline__ void tma_prefetch_map(const void* tmap) {
 // ---- tcgen05: tensor memory and the 5th-generation MMA --------------------
 
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
                : "memory");
 }
 __device__ __forceinline__ void tmem_relinquish() {
+  __syncwarp();
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -404,6 +412,7 @@ __device__ __forceinline__ void umma_commit(uint32_t mb) {
 // statement.
 __device__ __forceinline__ void tmem_ld8_sync(uint32_t taddr, float (&v)[8]) {
   uint32_t r[8];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
       "tcgen05.wait::ld.sync.aligned;"
@@ -421,6 +430,7 @@ __device__ __forceinline__ void tmem_ld8_sync(uint32_t taddr, float (&v)[8]) {
 __device__ __forceinline__ void tmem_ld8x4_sync(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3,
                                                 float (&v)[4][8]) {
   uint32_t r[32];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%32];\n\t"
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%33];\n\t"
@@ -441,6 +451,7 @@ __device__ __forceinline__ void tmem_ld8x4_sync(uint32_t t0, uint32_t t1, uint32
 // the values can be scheduled before they have arrived.
 __device__ __forceinline__ void tmem_ld16x2_sync(uint32_t ta, uint32_t tb, float (&va)[16], float (&vb)[16]) {
   uint32_t r[32];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%32];\n\t"
@@ -465,6 +476,7 @@ __device__ __forceinline__ void tmem_ld16x2_sync(uint32_t ta, uint32_t tb, float
 // waits for every tensor-memory load of the thread and then marks the
 // registers as redefined, so that the compiler schedules no use before it.
 __device__ __forceinline__ void tmem_ld16x2_issue(uint32_t ta, uint32_t tb, uint32_t (&r)[32]) {
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%32];\n\t"
@@ -475,6 +487,7 @@ __device__ __forceinline__ void tmem_ld16x2_issue(uint32_t ta, uint32_t tb, uint
       : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld_tie32(uint32_t (&r)[32]) {
+  __syncwarp();
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
   asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
   asm volatile("" : "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]));
@@ -485,6 +498,7 @@ __device__ __forceinline__ void tmem_wait_ld_tie32(uint32_t (&r)[32]) {
 // no use of the values can be scheduled before they have arrived.
 __device__ __forceinline__ void tmem_ld16_sync(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%16];\n\t"
@@ -500,6 +514,7 @@ __device__ __forceinline__ void tmem_ld16_sync(uint32_t taddr, float (&v)[16]) {
 // Store 16 consecutive 32-bit columns per lane (rows lane base + i) into
 // tensor memory; complete with tmem_wait_st().
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
+  __syncwarp();
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15, %16};" ::"r"(taddr),
@@ -510,7 +525,10 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) 
       "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
       : "memory");
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() {
+  __syncwarp();
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
 
 // Shared-memory matrix descriptor of a K-major bf16 tile written by TMA with
 // 128-byte swizzling: rows of 64 elements (128 B), 8-row groups 1024 B apart.
