@@ -410,7 +410,6 @@ __global__ void __launch_bounds__(rows_threads(XF, MT), 1)
         const int srow = tile_row(m) + lrow;
         const bool ok_row = (MT * (int)blockIdx.x + m) % a.kt_per_gate * kTileM + lrow < a.K;
         float v[16], w[16];
-        __syncwarp();
         tmem_ld16x2_sync(trow + m * 2 * BN + c0, trow + m * 2 * BN + BN + c0, v, w);
         float* p = a.P + (long long)(col0 + c0) * a.ldp + srow;
         const int nv = a.N - (col0 + c0);
@@ -741,12 +740,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
         for (int e = 0; e < 8; ++e) cp[e] = cpn[e];  // loaded before any store of this round
         load_c(c8 + 8, cpn);
-        __syncwarp();
         tmem_ld8x4_sync(trow + c8, trow + kGate + c8, trow + 2 * kGate + c8, trow + 3 * kGate + c8, y);
         if constexpr (kBoth) {
           float lo[4][8];
           const uint32_t tl = trow + NT + c8;
-          tmem_ld8x4_sync(tl, tl + kGate, tl + 2 * kGate, tl + 3 * kGate, lo);
+          tmem_ld8x4_sync<true>(tl, tl + kGate, tl + 2 * kGate, tl + 3 * kGate, lo);
 #pragma unroll
           for (int g = 0; g < 4; ++g)
 #pragma unroll

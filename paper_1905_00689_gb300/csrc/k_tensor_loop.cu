@@ -143,9 +143,10 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
 }
 
 // Two loads of 32 lanes x 8 consecutive columns and the wait for both in one statement.
+template <bool kTogether = false>
 __device__ __forceinline__ void tmem_ld8x2_sync(uint32_t ta, uint32_t tb, float (&va)[8], float (&vb)[8]) {
   uint32_t r[16];
-  __syncwarp();
+  if constexpr (!kTogether) __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n\t"
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n\t"
@@ -623,7 +624,8 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
     };
     // first stream of this thread's cells of stream tile s
     auto first_stream = [&](int s) { return (tb0 + s) * NT + (GP == 4 ? part * CW : zb * SO + part * CPT); };
-    // eight streams' sums of one gate over the segments [0, nseg) from column `col` (both planes' products)
+    // eight streams' sums of one gate over the segments [0, nseg) from column `col` (both planes' products); the
+    // caller's warp is together
     auto load_sums = [&](uint32_t col, int nseg, float (&v)[8]) {
 #pragma unroll
       for (int c = 0; c < 8; ++c) v[c] = 0.f;
@@ -632,11 +634,11 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
         float vh[8];
         if constexpr (MB) {
           float vl[8];
-          tmem_ld8x2_sync(col + i * seg, col + i * seg + NT, vh, vl);
+          tmem_ld8x2_sync<true>(col + i * seg, col + i * seg + NT, vh, vl);
 #pragma unroll
           for (int c = 0; c < 8; ++c) vh[c] += vl[c];
         } else {
-          tmem_ld8_sync(col + i * seg, vh);
+          tmem_ld8_sync<true>(col + i * seg, vh);
         }
 #pragma unroll
         for (int c = 0; c < 8; ++c) v[c] += vh[c];
@@ -650,7 +652,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       __syncwarp();
       if constexpr (GP == 4) {
         if (!MB && nseg == 1) {
-          tmem_ld8x4_sync(tc0, tc0 + dg, tc0 + 2 * dg, tc0 + 3 * dg, y);
+          tmem_ld8x4_sync<true>(tc0, tc0 + dg, tc0 + 2 * dg, tc0 + 3 * dg, y);
         } else {
 #pragma unroll
           for (int g = 0; g < 4; ++g) load_sums(tc0 + g * dg, nseg, y[g]);
@@ -666,6 +668,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
         const uint32_t buf =
             (setb ? L.rxb : L.rxa) + (u & 1u) * (a.share_rx ? max(a.rxa_bytes, a.rxb_bytes) : a.rxb_bytes);
         if (e == 0) mbar_arrive_expect_tx(rxb, (uint32_t)(4 * 128 * SO * 4));
+        __syncwarp();
         bool got = true;
 #pragma unroll
         for (int g = 0; g < GP; ++g)
@@ -817,7 +820,6 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
 #pragma unroll
             for (int c8 = 0; c8 < CW; c8 += 8) {
               float vh[8], vl[8];
-              __syncwarp();
               tmem_ld8x2_sync(tc0 + c8, tc0 + NT + c8, vh, vl);
               if (c8 + 8 == CW) {
                 tc_fence_before();
@@ -839,6 +841,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
               return (uint32_t)((row * kP + (p ^ x)) * 16);
             };
             if (e == 0) mbar_arrive_expect_tx(rxb, (uint32_t)(128 * NT * 4));
+            __syncwarp();
             const int owner = lrow / RS;
             const uint32_t peer = crank - (uint32_t)za + (uint32_t)owner;
             const uint32_t dst = mapa_shared(base + buf + (uint32_t)za * RS * NT * 4u, peer);
@@ -846,7 +849,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
 #pragma unroll
             for (int c8 = 0; c8 < CW; c8 += 8) {
               float vh[8], vl[8];
-              tmem_ld8x2_sync(tc0 + c8, tc0 + NT + c8, vh, vl);
+              tmem_ld8x2_sync<true>(tc0 + c8, tc0 + NT + c8, vh, vl);
               if (c8 + 8 == CW) {
                 tc_fence_before();
                 warp_arrive(handed);

@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(seq_threads(NS, NC), 1)
         for (int i8 = 0; i8 < SPW / 8; ++i8) {
           const int c8 = part * SPW + 8 * i8;
           float hl[16], v[8];  // the group's hi products, then its lo products
-          tmem_ld16_sync(trow + tAcc + 2 * c8, hl);
+          tmem_ld16_sync<true>(trow + tAcc + 2 * c8, hl);
 #pragma unroll
           for (int k8 = 0; k8 < 8; ++k8) v[k8] = hl[k8] + hl[8 + k8];
 #pragma unroll
@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(seq_threads(NS, NC), 1)
 #pragma unroll
               for (int g = 0; g < 4; ++g) {
                 float a0[16];
-                tmem_ld16_sync(tc0 + g * 2 * MT * NS, a0);
+                tmem_ld16_sync<true>(tc0 + g * 2 * MT * NS, a0);
 #pragma unroll
                 for (int k8 = 0; k8 < 8; ++k8) y[g][k8] = a0[k8] + a0[8 + k8];
               }
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(seq_threads(NS, NC), 1)
 #pragma unroll
               for (int g = 0; g < 4; g += 2) {
                 float a0[16], a1[16];
-                tmem_ld16x2_sync(tc0 + g * 2 * MT * NS, tc0 + (g + 1) * 2 * MT * NS, a0, a1);
+                tmem_ld16x2_sync<true>(tc0 + g * 2 * MT * NS, tc0 + (g + 1) * 2 * MT * NS, a0, a1);
 #pragma unroll
                 for (int k8 = 0; k8 < 8; ++k8) {
                   y[g][k8] = a0[k8] + a0[8 + k8];

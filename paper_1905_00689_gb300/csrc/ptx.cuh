@@ -47,6 +47,11 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
 // together.  A branch that only some lanes take (one lane arming a barrier,
 // lanes leaving a wait at different polls) does not by itself bring them back
 // together, so every wrapper of such an instruction starts with __syncwarp().
+// The tensor-memory loads take kTogether = true where the warp is together
+// already: between the load and the last warp-wide barrier, vote or load before
+// it are only branches that all its lanes take alike.  (In the cell loop of
+// tc_seq_kernel a barrier per load took 3.4% of a whole run: D=2048 H=1024 T=64
+// B=1024 K=8 440 -> 455 us.)
 __device__ __forceinline__ void cluster_sync_all() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -410,9 +415,10 @@ __device__ __forceinline__ void umma_commit(uint32_t mb) {
 
 // 32 lanes x 8 consecutive 32-bit columns and the wait for them in one
 // statement.
+template <bool kTogether = false>
 __device__ __forceinline__ void tmem_ld8_sync(uint32_t taddr, float (&v)[8]) {
   uint32_t r[8];
-  __syncwarp();
+  if constexpr (!kTogether) __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
       "tcgen05.wait::ld.sync.aligned;"
@@ -427,10 +433,11 @@ __device__ __forceinline__ void tmem_ld8_sync(uint32_t taddr, float (&v)[8]) {
 // the wait for them in one statement, so that no use of the values can be
 // scheduled before they have arrived: v[i][c] = column t_i + c of this
 // thread's row.
+template <bool kTogether = false>
 __device__ __forceinline__ void tmem_ld8x4_sync(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3,
                                                 float (&v)[4][8]) {
   uint32_t r[32];
-  __syncwarp();
+  if constexpr (!kTogether) __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%32];\n\t"
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%33];\n\t"
@@ -449,9 +456,10 @@ __device__ __forceinline__ void tmem_ld8x4_sync(uint32_t t0, uint32_t t1, uint32
 
 // Two 16-column loads and one wait for both in one statement, so that no use of
 // the values can be scheduled before they have arrived.
+template <bool kTogether = false>
 __device__ __forceinline__ void tmem_ld16x2_sync(uint32_t ta, uint32_t tb, float (&va)[16], float (&vb)[16]) {
   uint32_t r[32];
-  __syncwarp();
+  if constexpr (!kTogether) __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%32];\n\t"
@@ -496,9 +504,10 @@ __device__ __forceinline__ void tmem_wait_ld_tie32(uint32_t (&r)[32]) {
 // 32 lanes x 16 consecutive 32-bit columns of tensor memory (thread i of the
 // warp gets row lane base + i) and the wait for them in one statement, so that
 // no use of the values can be scheduled before they have arrived.
+template <bool kTogether = false>
 __device__ __forceinline__ void tmem_ld16_sync(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
-  __syncwarp();
+  if constexpr (!kTogether) __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%16];\n\t"

@@ -30,8 +30,27 @@ def test_aligned_instructions_follow_a_warp_barrier(name):
     for before, stmt in found:
         body = before[before.index("{") + 1:]
         # nothing but declarations and the barrier between the function's start and the instruction
-        rest = re.sub(r"uint32_t r\[\d+\];|__syncwarp\(\);", "", body)
+        rest = re.sub(r"uint32_t r\[\d+\];|if constexpr \(!kTogether\) |__syncwarp\(\);", "", body)
         assert "__syncwarp();" in body and rest.strip() == "", stmt[:80]
+
+
+# what only some lanes of a warp may do, or leave at different times
+LANE_BRANCH = re.compile(r"\b(?:e|lane|tid|threadIdx\.x) (?:==|<)|\b(?:elect_one|warp_arrive|mbar_wait_bounded|\w+_wait|wait_cta)\b")
+
+
+@pytest.mark.parametrize("name", [n for n in SOURCES if n.endswith(".cu")])
+def test_loads_without_a_barrier_are_reached_together(name):
+    """A load that leaves the barrier out (kTogether) follows a warp-wide
+    barrier or vote, or a load that has one, with no branch of single lanes
+    and no wait in between.  `load_sums` (k_tensor_loop.cu) passes the demand
+    on to its callers."""
+    with open(os.path.join(CSRC, name)) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    text = re.sub(r"auto load_sums = .*?\n    \};\n", "", text, flags=re.S)
+    for m in re.finditer(r"tmem_ld\w+<true>\(|\bload_sums\(", text):
+        last = [k for k in re.finditer(r"__syncwarp\(\);|__all_sync\(.*?\);|tmem_ld\w+\(.*?\);", text[:m.start()], re.S)][-1]
+        between = text[last.end():m.start()]
+        assert not LANE_BRANCH.search(between), (name, between)
 
 
 def test_the_wrappers_are_all_there():
