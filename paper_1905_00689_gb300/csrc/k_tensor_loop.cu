@@ -602,9 +602,12 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
     // c_{t-1} of this thread's cells: with one stream tile and no intermediate depths in registers across
     // the steps, otherwise in memory, by the parity of t (the depths of step t - 1 run during step t)
     const bool keep_c = nb <= 1 && ndep == 0;
+    const bool defer = a.defer_depths != 0 && ndep > 0 && nb > 0;  // a step's depths run during the next step
     float cp[CPT];
-    auto load_c = [&](int t, int n0) {
-      const float* src = t == 0 ? a.c0 : (t & 1) ? a.c_state1 : a.c_state;
+    // (c_{-1} = c0: the full depth reads it from the caller and keeps a copy for the depths that run after the
+    // step's outputs are written, because the caller may pass one buffer as c0 and as an output)
+    auto load_c = [&](int t, int n0, bool depths) {
+      const float* src = (t & 1) ? a.c_state1 : (t > 0 || depths) ? a.c_state : a.c0;
 #pragma unroll
       for (int c = 0; c < CPT; ++c) cp[c] = (unit_ok && n0 + c < B && src != nullptr) ? src[(n0 + c) * H + j] : 0.f;
     };
@@ -753,6 +756,12 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
             for (int c = 0; c < CPT; ++c)
               if (n0 + c < B) o[(n0 + c) * H] = hv[c];
           }
+          if (defer && t == 0) {
+            float* o = a.c_state + j;
+#pragma unroll
+            for (int c = 0; c < CPT; ++c)
+              if (n0 + c < B) o[(n0 + c) * H] = cp[c];
+          }
           if (!keep_c) {
             float* o = ((t & 1) ? a.c_state : a.c_state1) + j;
 #pragma unroll
@@ -776,13 +785,12 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       bool fail = false;
 #pragma unroll 1
       for (int s = 0; s < nb && !fail; ++s) {
-        load_c(t, first_stream(s));
+        load_c(t, first_stream(s), true);
         fail = !run_sets(t, s, region, 1, ndep + 1);
         if (++region == regs_b) region = 0;
       }
       return !block_or_named(1, EPI, fail);
     };
-    const bool defer = a.defer_depths != 0 && ndep > 0 && nb > 0;
     bool ok = true;
     // h_{-1} = h0 (or zero) of this CTA's units and streams
     for (int s = 0; s < nb && ok; ++s) {
@@ -890,7 +898,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       reg_first = pb.slot;
 #pragma unroll 1
       for (int s = 0; s < nb && ok; ++s) {
-        if (t == 0 || !keep_c) load_c(t, first_stream(s));
+        if (t == 0 || !keep_c) load_c(t, first_stream(s), false);
         const bool got = __all_sync(0xffffffffu, mbar_wait_bounded<false>(acc_b + 8u * pb.slot, pb.parity, limit, err));
         tc_fence_after();
         bool good = got && run_sets(t, s, pb.slot, 0, 1);

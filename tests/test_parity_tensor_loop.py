@@ -143,6 +143,39 @@ def test_bounded_wait_reports_timeout(cuda_device, H, K):
     assert np.array_equal(out.double().cpu().numpy(), ref["h"])
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("T", [1, 2])
+@pytest.mark.parametrize("H,B,K,cps", [
+    (136, 40, 40, [10, 32]),    # all gates in a CTA
+    (512, 70, 200, [64, 100]),  # one gate per CTA
+    (512, 40, 902, [451]),      # segments
+    (1024, 300, 128, [64]),     # several stream tiles per CTA
+])
+def test_state_in_place(cuda_device, H, B, K, cps, T):
+    """The same buffers as initial and final state (a caller that resumes one
+    call after another): every output as with separate buffers."""
+    import torch
+    D = 40
+    gates = _gates(H, D + H, K, 50, 8600 + H + K)
+    rng = np.random.default_rng(86)
+    x = torch.from_numpy(draw_inputs(T, B, D, "uniform", 86).astype(np.float32)).cuda()
+    h0, c0 = (torch.from_numpy(rng.standard_normal((1, B, H)).astype(np.float32)).cuda() for _ in range(2))
+    m = LSTMApprox(1, [D], H, K, B, "bf16")
+    m.set_layer(0, gates)
+    res = []
+    for in_place in (False, True):
+        h_in, c_in = h0.clone(), c0.clone()
+        c_out = c_in if in_place else torch.empty_like(c_in)
+        out = h_in if in_place and T == 1 else torch.empty(T, B, H, device="cuda")
+        ck = torch.empty(2, len(cps), T, B, H, device="cuda")
+        m.run(x, K, out, h0=h_in, c0=c_in, out_c=c_out, checkpoints=cps, ckpt_h=ck[0], ckpt_c=ck[1])
+        m.sync()
+        assert m.query(Q_TENSOR_LOOP) == 1
+        res.append((out, c_out, ck))
+    for apart, same in zip(*res):
+        assert torch.equal(apart, same)
+
+
 @pytest.mark.parametrize("H,B,K,cps,loop", [
     (512, 256, 512, [], 1), (512, 256, 32, [], 0),             # K <= 32 at H = 512: one launch per stream tile
     (600, 100, 32, [10], 1), (2048, 64, 1024, [16, 256], 1),
