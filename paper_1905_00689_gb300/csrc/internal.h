@@ -431,6 +431,7 @@ struct TcLoopPlan {
   int cut_k[kLoopMaxCuts];
   int stream_segs;           // 1: the segments take the accumulator regions in turn (no intermediate depths)
   int dep_segs[kMaxCheckpoints];  // segments that depth i sums
+  int split_depths;          // 1: an intermediate depth lies inside a 16-term slice
 };
 struct TcLoopArgs : TcLoopPlan {
   int H, K, Ks, B, T;

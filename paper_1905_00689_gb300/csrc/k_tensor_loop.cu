@@ -192,6 +192,40 @@ __device__ __forceinline__ bool wait_counter(const unsigned* c, unsigned target,
   return true;
 }
 
+// One unit's cell of one stream at the intermediate depth kd from the factor and the stored tau' pair, in place
+// of sums in which a tau' past the depth that is not finite met a zero of U (see run_sets).  `u`, `tau`: the unit's
+// and the stream's first gate; gate g follows at u + g gate_u and tau + g Ks.
+__device__ __noinline__ void depth_cell(const __nv_bfloat16* u, long long gate_u, const __nv_bfloat16* tau,
+                                        long long tau_plane, int Ks, int kd, const float* bias, int H, float c_prev,
+                                        float* h_out, float* c_out) {
+  float y[4];
+#pragma unroll 1
+  for (int g = 0; g < 4; ++g) {
+    float acc = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < kd; k += 8) {
+      const uint4 wu = __ldg(reinterpret_cast<const uint4*>(u + g * gate_u + k));
+      const uint4 wh = __ldcg(reinterpret_cast<const uint4*>(tau + g * Ks + k));
+      const uint4 wl = __ldcg(reinterpret_cast<const uint4*>(tau + tau_plane + g * Ks + k));
+      const uint32_t* pu = reinterpret_cast<const uint32_t*>(&wu);
+      const uint32_t* ph = reinterpret_cast<const uint32_t*>(&wh);
+      const uint32_t* pl = reinterpret_cast<const uint32_t*>(&wl);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        auto value = [&](const uint32_t* w) {
+          return __uint_as_float((e & 1) != 0 ? w[e >> 1] & 0xFFFF0000u : w[e >> 1] << 16);
+        };
+        if (k + e < kd) acc = fmaf(value(pu), value(ph) + value(pl), acc);
+      }
+    }
+    y[g] = acc + bias[g * H];
+  }
+  float hh, cc;
+  lstm_cell_s(y[0], y[1], y[2], y[3], c_prev, hh, cc);
+  if (h_out != nullptr) *h_out = hh;
+  if (c_out != nullptr) *c_out = cc;
+}
+
 // Position in the stage ring: slot and phase parity, advanced without divisions (one thread issues
 // everything, so its instructions are on the path of every step).
 struct RingPos {
@@ -205,7 +239,9 @@ struct RingPos {
   }
 };
 
-template <int NT, int GP, bool MB>
+// SD: an intermediate depth lies inside a 16-term slice (what that takes in the epilogue is left out of the other
+// shapes' kernels: with it H = 1024, B = 1024, K = 128 without depths took 1132 us a run instead of 943)
+template <int NT, int GP, bool MB, bool SD>
 __global__ void __launch_bounds__(loop_threads(NT), 1)
     tc_loop_kernel(const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmu,
                    const __grid_constant__ CUtensorMap tmh, const __grid_constant__ CUtensorMap tmt, TcLoopArgs a) {
@@ -611,18 +647,62 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
 #pragma unroll
       for (int c = 0; c < CPT; ++c) cp[c] = (unit_ok && n0 + c < B && src != nullptr) ? src[(n0 + c) * H + j] : 0.f;
     };
-    auto store_depth = [&](int jj, int t, int n0, const float (&h)[CPT], const float (&c)[CPT]) {
+    auto store_depth = [&](int jj, int t, int n0, const float (&h)[CPT], const float (&c)[CPT], unsigned skip) {
       if (!unit_ok) return;
       const long long o = (long long)jj * a.ck_stride + ((long long)t * B + n0) * H + j;
       if (a.ckpt_h) {
 #pragma unroll
         for (int i = 0; i < CPT; ++i)
-          if (n0 + i < B) a.ckpt_h[o + i * H] = h[i];
+          if (n0 + i < B && (skip >> i & 1u) == 0u) a.ckpt_h[o + i * H] = h[i];
       }
       if (a.ckpt_c) {
 #pragma unroll
         for (int i = 0; i < CPT; ++i)
-          if (n0 + i < B) a.ckpt_c[o + i * H] = c[i];
+          if (n0 + i < B && (skip >> i & 1u) == 0u) a.ckpt_c[o + i * H] = c[i];
+      }
+    };
+    // Depths inside a 16-term slice (SD): the products of the slice's terms past the depth have a zero
+    // of U, and a tau' of such a term that is not finite makes them NaN (its pair's lo half is one even for an
+    // infinity).  The full depth's sums are then NaN too, in all units of the stream.  So: cells (bits) whose sums
+    // are NaN get their depths from depth_cell at the full depth of the step, while tau'_t is still in memory
+    // (its next value waits for this CTA's h_t), and the depths' own pass leaves out what is NaN there.
+    auto any_nan = [&](const float (&y)[4][CPT]) -> bool {
+      uint64_t s2 = f32x2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < CPT; c += 2)
+#pragma unroll
+        for (int g = 0; g < 4; ++g) s2 = add2(s2, f32x2(y[g][c], y[g][c + 1]));
+      float s0, s1;
+      f32x2_split(s2, s0, s1);
+      const float sum = s0 + s1;
+      return sum != sum;
+    };
+    auto nan_cells = [&](const float (&y)[4][CPT], int n0) -> unsigned {
+      unsigned m = 0u;
+#pragma unroll
+      for (int c = 0; c < CPT; ++c) {
+        const float sum = (y[0][c] + y[1][c]) + (y[2][c] + y[3][c]);
+        if (sum != sum && unit_ok && n0 + c < B) m |= 1u << c;
+      }
+      return m;
+    };
+    bool nan_seen = false;  // in a full depth of this thread's cells so far
+    auto exact_depths = [&](unsigned cells, int t, int s, int n0) {
+      unsigned seen;  // (every row tile's tau'_t has been released to this counter)
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.tau_count + 32 * (tb0 + s)) : "memory");
+#pragma unroll 1
+      for (; cells != 0u; cells &= cells - 1u) {
+        const int c = __ffs(cells) - 1;
+        float cv = cp[0];
+#pragma unroll
+        for (int i = 1; i < CPT; ++i) cv = i == c ? cp[i] : cv;
+#pragma unroll 1
+        for (int d = 0; d < ndep; ++d) {
+          const long long o = (long long)d * a.ck_stride + ((long long)t * B + n0 + c) * H + j;
+          depth_cell(a.U + (long long)j * a.Ks, (long long)H * a.Ks, a.tau + (long long)(n0 + c) * a.ldt, a.tau_plane,
+                     a.Ks, a.cut_k[a.dep_segs[d] - 1], a.bias + j, H, cv, a.ckpt_h ? a.ckpt_h + o : nullptr,
+                     a.ckpt_c ? a.ckpt_c + o : nullptr);
+        }
       }
     };
     // first stream of this thread's cells of stream tile s
@@ -647,6 +727,36 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
         for (int c = 0; c < 8; ++c) v[c] += vh[c];
       }
     };
+    // role B's receive buffer of its exchange number u
+    auto receive_buf = [&](uint32_t u) {
+      return (setb ? L.rxb : L.rxa) + (u & 1u) * (a.share_rx ? max(a.rxa_bytes, a.rxb_bytes) : a.rxb_bytes);
+    };
+    auto read_received = [&](uint32_t buf, float (&y)[4][CPT]) {
+      const float* rb = reinterpret_cast<const float*>(gb_ + buf) + part * CPT;
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int c = 0; c < CPT; c += 2) {
+          const float2 f = *reinterpret_cast<const float2*>(rb + (g * 128 + lrow) * SO + c);
+          y[g][c] = f.x;
+          y[g][c + 1] = f.y;
+        }
+    };
+    // the four gates' sums as this CTA holds them: in tensor memory (GP = 4) or in the receive buffer of the last
+    // exchange; the caller's warp is together
+    auto read_sums = [&](int region, int nseg, float (&y)[4][CPT]) {
+      if constexpr (GP == 4) {
+        const uint32_t tc0 = trow + a.acc_b + (uint32_t)region * reg_segs * seg + part * CW;
+        if (!MB && nseg == 1) {
+          tmem_ld8x4_sync<true>(tc0, tc0 + dg, tc0 + 2 * dg, tc0 + 3 * dg, y);
+        } else {
+#pragma unroll
+          for (int g = 0; g < 4; ++g) load_sums(tc0 + g * dg, nseg, y[g]);
+        }
+      } else {
+        read_received(receive_buf(rx_use[setb] - 1u), y);
+      }
+    };
     // the gate sums y over nseg segments of accumulator region `region`; with several CTAs
     // per unit tile (GP < 4) each sends its gates' sums to the owners of the streams and takes what they
     // sent; `last`: the accumulators are not read again
@@ -654,12 +764,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       const uint32_t tc0 = trow + a.acc_b + (uint32_t)region * reg_segs * seg + part * CW;
       __syncwarp();
       if constexpr (GP == 4) {
-        if (!MB && nseg == 1) {
-          tmem_ld8x4_sync<true>(tc0, tc0 + dg, tc0 + 2 * dg, tc0 + 3 * dg, y);
-        } else {
-#pragma unroll
-          for (int g = 0; g < 4; ++g) load_sums(tc0 + g * dg, nseg, y[g]);
-        }
+        read_sums(region, nseg, y);
         if (last) {
           tc_fence_before();
           warp_arrive(drain_b + 8u * region);
@@ -668,8 +773,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
       } else {
         const uint32_t u = rx_use[setb]++;
         const uint32_t rxb = rx0 + 16u * setb + 8u * (u & 1u);
-        const uint32_t buf =
-            (setb ? L.rxb : L.rxa) + (u & 1u) * (a.share_rx ? max(a.rxa_bytes, a.rxb_bytes) : a.rxb_bytes);
+        const uint32_t buf = receive_buf(u);
         if (e == 0) mbar_arrive_expect_tx(rxb, (uint32_t)(4 * 128 * SO * 4));
         __syncwarp();
         bool got = true;
@@ -708,15 +812,7 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           warp_arrive(drain_b + 8u * (stream ? pb.slot : region));
         }
         got = __all_sync(0xffffffffu, mbar_wait_bounded<true>(rxb, (u >> 1) & 1u, limit, err)) && got;
-        const float* rb = reinterpret_cast<const float*>(gb_ + buf) + part * CPT;
-#pragma unroll
-        for (int g = 0; g < 4; ++g)
-#pragma unroll
-          for (int c = 0; c < CPT; c += 2) {
-            const float2 f = *reinterpret_cast<const float2*>(rb + (g * 128 + lrow) * SO + c);
-            y[g][c] = f.x;
-            y[g][c + 1] = f.y;
-          }
+        read_received(buf, y);
         return got;
       }
     };
@@ -734,16 +830,28 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
           if (set == 0) publish(true, a.h_count, true);  // the barrier where the block's other warps wait
           break;
         }
+        unsigned nans = 0u;
+        if constexpr (SD) {
+          if (set > 0) {
+            if (nan_seen) nans = nan_cells(y, n0);
+          } else if (__any_sync(0xffffffffu, any_nan(y))) {
+            nans = nan_cells(y, n0);
+            nan_seen = nan_seen || nans != 0u;
+            exact_depths(nans, t, s, n0);
+            __syncwarp();
+            read_sums(region, ncut + 1, y);
+          }
+        }
         lstm_cells_s(y, bias, cp, hv, cv);
         if (set > 0) {
-          store_depth(set - 1, t, n0, hv, cv);
+          store_depth(set - 1, t, n0, hv, cv, nans);
           continue;
         }
 #pragma unroll
         for (int c = 0; c < CPT; c += 2) store_h2(a.h_bf16, a.ldh, a.h_plane, n0 + c, hv[c], hv[c + 1]);
         if (!publish(false, a.h_count + 32 * (tb0 + s), false)) return false;
         // then what nothing waits for
-        for (int jj = ndep; jj < a.ck_n; ++jj) store_depth(jj, t, n0, hv, cv);  // depths of at least K
+        for (int jj = ndep; jj < a.ck_n; ++jj) store_depth(jj, t, n0, hv, cv, 0u);  // depths of at least K
         if (a.seq_bf16) {
           __nv_bfloat16* sq = a.seq_bf16 + (long long)t * B * a.ldh;
 #pragma unroll
@@ -940,10 +1048,10 @@ __global__ void __launch_bounds__(loop_threads(NT), 1)
 }
 
 
-template <int NT, int GP, bool MB>
+template <int NT, int GP, bool MB, bool SD>
 cudaError_t launch_loop_t(const TcMap& V, const TcMap& U, const TcMap& Hm, const TcMap& Taum, const TcLoopPlan& p,
                           const TcLoopArgs& a, cudaStream_t s, bool* resident) {
-  auto kern = tc_loop_kernel<NT, GP, MB>;
+  auto kern = tc_loop_kernel<NT, GP, MB, SD>;
   // per thread and device: the shared-memory limit, and the cluster sizes and sizes of grids known to be resident
   static thread_local unsigned long long ready = 0;
   static thread_local struct {
@@ -1029,6 +1137,7 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     }
     ++p.ndep;
   }
+  p.split_depths = pieces > 0 ? 1 : 0;
   // The segments: up to each depth, and for K > 512 no longer than kLoopSegTerms, because the rounding of a
   // long running sum adds up.  Error of h against 64 bits, one accumulator / segments / the two launches (which
   // split K over CTAs): H = 512, B = 16, K = 902 4.5e-6 / 3.3e-6 / 3.4e-6; H = 256, B = 64, K = 1000
@@ -1146,8 +1255,10 @@ cudaError_t launch_tc_loop(const TcMap& V, const TcMap& U, const TcMap& Hm, cons
                            const TcLoopArgs& args, cudaStream_t s, bool* resident) {
   TcLoopArgs a = args;
   static_cast<TcLoopPlan&>(a) = p;
-#define LA_LOOP(NT_, GP_, MB_) \
-  if (p.nt == NT_ && p.gp == GP_ && (p.mb != 0) == MB_) return launch_loop_t<NT_, GP_, MB_>(V, U, Hm, Taum, p, a, s, resident);
+#define LA_LOOP(NT_, GP_, MB_)                                                                         \
+  if (p.nt == NT_ && p.gp == GP_ && (p.mb != 0) == MB_)                                               \
+    return p.split_depths ? launch_loop_t<NT_, GP_, MB_, true>(V, U, Hm, Taum, p, a, s, resident)     \
+                          : launch_loop_t<NT_, GP_, MB_, false>(V, U, Hm, Taum, p, a, s, resident);
   LA_LOOP(16, 4, false) LA_LOOP(16, 1, false) LA_LOOP(32, 4, false) LA_LOOP(32, 1, false)
   LA_LOOP(16, 4, true) LA_LOOP(16, 1, true) LA_LOOP(32, 4, true) LA_LOOP(32, 1, true)
 #undef LA_LOOP

@@ -176,6 +176,35 @@ def test_state_in_place(cuda_device, H, B, K, cps, T):
         assert torch.equal(apart, same)
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,B,K,cps,term", [
+    (72, 20, 48, [10, 45], 12),      # all gates in a CTA; the term shares the first depth's slice
+    (72, 20, 48, [10, 32, 45], 46),  # ... the last depth's; the others end before it
+    (1024, 300, 128, [20, 64], 21),  # several stream tiles per CTA
+    (512, 40, 200, [100, 133], 143),  # one gate per CTA
+    (512, 40, 902, [451, 455], 453),  # segments; one depth before the term, one past it
+])
+def test_depths_ignore_later_terms_that_are_not_finite(cuda_device, H, B, K, cps, term):
+    """A term whose coefficient is infinite leaves the depths that end before
+    it what they are without it, also inside its 16-term slice; everything
+    agrees with the two-launches-per-step kernels, which stop at the depth."""
+    D, T = 32, 3
+    gates = _gates(H, D + H, K, 50, 8700 + H + K)
+    x = draw_inputs(T, B, D, "uniform", 87)
+    plain, _ = run_gpu([gates], x, K, dtype="bf16", checkpoints=cps)
+    gates[1]["sigma"] = gates[1]["sigma"].copy()
+    gates[1]["sigma"][term] = np.inf
+    got, m = run_gpu([gates], x, K, dtype="bf16", checkpoints=cps)
+    assert m.query(Q_TENSOR_LOOP) == 1
+    step, m2 = run_gpu([gates], x, K, dtype="bf16", checkpoints=cps, tensor_seq=1)
+    assert m2.query(Q_TENSOR_LOOP) == 0
+    for k in got:
+        assert np.isfinite(step[k]).all() and np.abs(got[k] - step[k]).max() <= 4e-4 * np.abs(step[k]).max(), k
+    for i, c in enumerate(cps):
+        if c <= term:  # the first step starts from the same state
+            assert np.abs(got["ckpt_h"][i, 0] - plain["ckpt_h"][i, 0]).max() <= 1e-5
+
+
 @pytest.mark.parametrize("H,B,K,cps,loop", [
     (512, 256, 512, [], 1), (512, 256, 32, [], 0),             # K <= 32 at H = 512: one launch per stream tile
     (600, 100, 32, [10], 1), (2048, 64, 1024, [16, 256], 1),
