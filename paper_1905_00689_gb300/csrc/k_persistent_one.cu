@@ -49,8 +49,8 @@ constexpr int kStepsPerPass = 8;  // timesteps per read of a row's x part
 
 struct OneDev {
   int LA, LB;  // lanes per coefficient row, per gate row (powers of two)
-  int KP;      // stride of a gate's tau' in shared memory
-  int HP;      // h buffer length
+  int KP;      // stride of a gate's tau' in shared memory; the last quad stays zero
+  int HP;      // h buffer length; the last quad stays zero
 };
 
 // Sum over the 2^lg lanes that differ in the low lg bits of the lane index.
@@ -216,11 +216,13 @@ __global__ void __launch_bounds__(NTH, 1) persistent_one_kernel(PersistentArgs a
   float p_next = 0.f;
   if (row_ok && la == 0) p_next = pr.mode != 0 ? P_s[r] : __ldcg(Pg);
   const int base = lane & ~(4 * p.LB - 1);  // the first of the unit's 4 LB lanes
-  int qa[VQ], qb[VQ];                 // shared-memory offsets of this lane's quads of h and tau'
+  // shared-memory offsets of this lane's quads of h and tau'; past the row they read the zero quad (the lane's
+  // factor values are zero there, but zero times an infinity is not)
+  int qa[VQ], qb[VQ];
 #pragma unroll
   for (int i = 0; i < VQ; ++i) {
-    qa[i] = 4 * min(la + p.LA * i, p.HP / 4 - 1);
-    qb[i] = g_b * p.KP + 4 * min(lb + p.LB * i, p.KP / 4 - 1);
+    qa[i] = la + p.LA * i < HQ ? 4 * (la + p.LA * i) : p.HP - 4;
+    qb[i] = g_b * p.KP + (4 * (lb + p.LB * i) < K ? 4 * (lb + p.LB * i) : p.KP - 4);
   }
   int kcut[4];  // the first round's depths (K: the full sums)
 #pragma unroll
@@ -354,9 +356,9 @@ bool plan_persistent_one(int H, int K, bool gathers, PersistentOnePlan* out) {
   }
   return false;
 found:
-  p.HP = (H + 3) / 4 * 4;
+  p.HP = (H + 3) / 4 * 4 + 4;
   // the four gates' rows eight banks apart, so that the 16-byte reads of a unit's lanes do not collide
-  p.KP = ((K + 3) / 4 * 4 + 23) / 32 * 32 + 8;
+  p.KP = ((K + 3) / 4 * 4 + 4 + 23) / 32 * 32 + 8;
   *out = p;
   return true;
 }

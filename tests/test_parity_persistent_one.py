@@ -52,20 +52,38 @@ def test_one_cta_kernel(cuda_device, D, H, T, B, K, nz, cps, L, launches):
 
 @pytest.mark.gpu
 def test_depths_ignore_later_terms_that_are_not_finite(cuda_device):
-    """A term whose x part meets an infinite input is not finite; depths below
-    it stay what they are without it."""
+    """A term whose coefficient is infinite leaves the depths that end before
+    it what they are without it."""
     D, H, T, K = 16, 16, 1, 6
     gates = [draw_factor_set(H, D + H, K, D, 9300 + g) for g in range(4)]
-    for g in gates:
-        g["idx"][:] = np.arange(1, D + 1)
-        g["idx"][K - 1] = np.arange(0, D)  # only the last term keeps column 0
     x = draw_inputs(T, 1, D, "uniform", 93)
-    x[0, 0, 0] = np.inf
+    plain, _ = run_gpu([gates], x, K, checkpoints=[2, 5])
+    for g in gates:
+        g["sigma"] = g["sigma"].copy()
+        g["sigma"][K - 1] = np.inf
     got, m = run_gpu([gates], x, K, checkpoints=[2, 5])
-    ref, _ = run_gpu([gates], x, K, checkpoints=[2, 5], variant=1)
     assert m.query(Q_PERSISTENT_VARIANT) == 3
-    assert np.array_equal(np.isfinite(got["ckpt_h"]), np.isfinite(ref["ckpt_h"]))
-    assert np.array_equal(np.isfinite(got["h"]), np.isfinite(ref["h"]))
+    assert not np.array_equal(got["h"], plain["h"])
+    for k in ("ckpt_h", "ckpt_c"):
+        assert np.isfinite(plain[k]).all() and np.array_equal(got[k], plain[k]), k
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,K,term", [(8, 8, 5), (8, 40, 37), (4, 104, 101), (64, 8, 7)])
+def test_lanes_past_a_row_meet_no_infinity(cuda_device, H, K, term):
+    """Lanes without values of their own add nothing, also where the row's
+    last coefficients are infinite: the gate saturates, as for a very large
+    coefficient."""
+    D, T = 12, 2
+    gates = [draw_factor_set(H, D + H, K, 10, 9350 + g) for g in range(4)]
+    gates[2]["sigma"] = gates[2]["sigma"].copy()
+    x = draw_inputs(T, 1, D, "uniform", 94)
+    gates[2]["sigma"][term] = 1e30
+    ref = oracle_run([gates], x, K, checkpoints=[4])
+    gates[2]["sigma"][term] = np.inf
+    got, m = run_gpu([gates], x, K, checkpoints=[4])
+    assert m.query(Q_PERSISTENT_VARIANT) == 3
+    assert_parity(got, ref, FP32_TOL)
 
 
 @pytest.mark.parametrize("H,K,one", [(64, 16, 1), (64, 32, 1), (64, 33, 0), (128, 16, 1), (128, 17, 0), (129, 4, 0),
