@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/lstm_approx.h"
+#include "device_set.h"
 
 namespace lstm_approx_impl {
 
@@ -17,6 +18,18 @@ struct Checkpoints {
   int n;
   int k[kMaxCheckpoints];
 };
+
+// Runs `prepare` (function attributes of a kernel) unless `done`, the calling
+// thread's set for that kernel, already has the current device.
+template <typename F>
+cudaError_t once_per_device(DeviceSet* done, F prepare) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || done->has(dev)) return e;
+  e = prepare();
+  if (e == cudaSuccess) done->add(dev);
+  return e;
+}
 
 // Opaque storage of one CUtensorMap (128 bytes, 64-byte aligned).
 struct alignas(64) TcMap {

@@ -536,15 +536,13 @@ cudaError_t launch_ag_t(const AgPlan& p, size_t smem, const PersistentArgs& a, c
   attr[1].val.programmaticStreamSerializationAllowed = a.proj_flags == nullptr ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  static thread_local bool attrs_set = false;
+  static thread_local DeviceSet ready;
   static thread_local unsigned long long checked[16] = {};
-  if (!attrs_set) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    attrs_set = true;
-  }
+  const cudaError_t ea = once_per_device(&ready, [&] {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (ea != cudaSuccess) return ea;
   const unsigned long long key = (static_cast<unsigned long long>(smem) << 8) | static_cast<unsigned>(p.CS);
   bool seen = false;
   for (unsigned long long k : checked) seen |= (k == key);

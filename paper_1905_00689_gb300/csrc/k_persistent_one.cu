@@ -386,16 +386,10 @@ namespace {
 template <int NTH, int VQ>
 cudaError_t launch_one_t(const PersistentOnePlan& p, const PersistentArgs& a, const OneProj& pr, cudaStream_t s) {
   auto kern = persistent_one_kernel<NTH, VQ>;
-  static thread_local unsigned long long ready = 0;  // bit d: the shared-memory limit is set on device d
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-  if (bit == 0 || (ready & bit) == 0) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    ready |= bit;
-  }
+  static thread_local DeviceSet ready;
+  const cudaError_t ea = once_per_device(
+      &ready, [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); });
+  if (ea != cudaSuccess) return ea;
   OneDev d;
   d.LA = p.LA;
   d.LB = p.LB;

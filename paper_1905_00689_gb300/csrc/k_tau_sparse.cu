@@ -100,14 +100,12 @@ int tau_sparse_max_h() { return 1280; }  // 160 KB of h besides the 35 KB of sta
 
 cudaError_t launch_tau_sparse(const TauSparseArgs& a, cudaStream_t s) {
   const size_t smem = tau_sparse_smem(a.H);
-  static thread_local bool attr = false;
-  if (!attr) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(tau_sparse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tau_sparse_smem(tau_sparse_max_h()));
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static thread_local DeviceSet ready;
+  const cudaError_t ea = once_per_device(&ready, [] {
+    return cudaFuncSetAttribute(tau_sparse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)tau_sparse_smem(tau_sparse_max_h()));
+  });
+  if (ea != cudaSuccess) return ea;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((4 * a.Rp + kRowsPerCta - 1) / kRowsPerCta, (a.B + kStreams - 1) / kStreams);
   cfg.blockDim = dim3(kWarpsPerCta * 32);

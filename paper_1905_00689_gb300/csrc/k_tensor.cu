@@ -951,13 +951,11 @@ size_t gates_smem() {
 template <int BN, int S, bool XF = false, int MT = 1>
 cudaError_t launch_rows_t(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, int n_cols, cudaStream_t s) {
   auto kern = tc_rows_kernel<BN, S, XF, MT>;
-  static thread_local bool attr = false;
+  static thread_local DeviceSet ready;
   const size_t smem = rows_smem<BN, S, XF, MT>();
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  const cudaError_t ea = once_per_device(
+      &ready, [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+  if (ea != cudaSuccess) return ea;
   static_assert((size_t)kTileM * (BN + 4) * 4 <= (size_t)S * (kABytes + 2 * BN * kTileK * 2),
                 "a split's receive buffer fits over the stage ring");
   const int sk = (!XF && a.sk > 1) ? a.sk : 1;
@@ -988,13 +986,11 @@ cudaError_t launch_rows_t(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, 
 template <int NT, int S, bool SPLIT>
 cudaError_t launch_gates_t(const TcMap& U, const TcMap& Tau, const TcGatesArgs& a, cudaStream_t s) {
   auto kern = tc_gates_kernel<NT, S, SPLIT>;
-  static thread_local bool attr = false;
+  static thread_local DeviceSet ready;
   const size_t smem = gates_smem<NT, S, SPLIT>();
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  const cudaError_t ea = once_per_device(
+      &ready, [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+  if (ea != cudaSuccess) return ea;
   const cudaError_t e =
       launch_pdl_block(kern, dim3((a.H + kTileM - 1) / kTileM, (a.B + NT - 1) / NT, a.ks), dim3(kTcThreads), smem, s,
                        *reinterpret_cast<const CUtensorMap*>(U.bytes),

@@ -1053,20 +1053,17 @@ cudaError_t launch_loop_t(const TcMap& V, const TcMap& U, const TcMap& Hm, const
                           const TcLoopArgs& a, cudaStream_t s, bool* resident) {
   auto kern = tc_loop_kernel<NT, GP, MB, SD>;
   // per thread and device: the shared-memory limit, and the cluster sizes and sizes of grids known to be resident
-  static thread_local unsigned long long ready = 0;
+  static thread_local DeviceSet ready;
   static thread_local struct {
     int dev, cs, ctas;
     size_t smem;
   } seen[16] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = once_per_device(
+        &ready, [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); });
   if (e != cudaSuccess) return e;
-  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-  if (bit == 0 || (ready & bit) == 0) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e != cudaSuccess) return e;
-    ready |= bit;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.ctas);
   cfg.blockDim = dim3(loop_threads(NT));

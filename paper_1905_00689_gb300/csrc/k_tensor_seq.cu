@@ -583,12 +583,10 @@ template <int NS, int MT, int NC = 1>
 cudaError_t launch_seq_t(const TcMap& Vh_p, const TcMap& U64, const TcSeqArgs& a, cudaStream_t s) {
   auto kern = tc_seq_kernel<NS, MT, NC>;
   const size_t smem = seq_layout(NS, MT, NC, 128).total;  // the largest layout of this kernel
-  static thread_local bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static thread_local DeviceSet ready;
+  const cudaError_t ea = once_per_device(
+      &ready, [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
+  if (ea != cudaSuccess) return ea;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.cs, (a.B + NC * NS - 1) / (NC * NS));
   cfg.blockDim = dim3(seq_threads(NS, NC));

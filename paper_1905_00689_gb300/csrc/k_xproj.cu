@@ -371,18 +371,11 @@ int xproj_split(int row_tiles, int col_chunks, int D, int max_split) {
 // (XprojSignal) cannot wait for.
 template <typename TF, int NC>
 cudaError_t prepare_nc() {
-  static thread_local unsigned long long done = 0;  // bit d: device d prepared
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-  if (bit == 0 || (done & bit) == 0) {
-    e = cudaFuncSetAttribute(xproj_kernel<TF, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes<TF, NC>());
-    if (e != cudaSuccess) return e;
-    done |= bit;
-  }
-  return cudaSuccess;
+  static thread_local DeviceSet done;
+  return once_per_device(&done, [] {
+    return cudaFuncSetAttribute(xproj_kernel<TF, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem_bytes<TF, NC>());
+  });
 }
 
 template <typename TF>
