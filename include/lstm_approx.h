@@ -311,7 +311,14 @@ enum lstm_approx_option_key {
                                masked-dense tau'; else one launch over all
                                tiles for all T where the factors and the
                                streams fit the GPU's CTAs: H <= 2048,
-                               K <= 1024), 1 = two launches per timestep */
+                               K <= 1024), 1 = two launches per timestep.
+                               The launch over all tiles is cooperative: its
+                               up to 148 CTAs start together, once the other
+                               kernels on the GPU have left that many SMs,
+                               however long that takes (the wait limit
+                               counts from the start).  The two launches per
+                               timestep run on whatever SMs are free: take 1
+                               where long kernels share the GPU. */
   LSTM_APPROX_OPT_LAUNCH_ORDER = 9 /* batch-1 fp32 path with the per-unit-block
                                kernel: 0 = automatic (the recurrence is
                                launched before its input projection and
