@@ -17,9 +17,7 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 }
 
 // True in exactly one thread of the (converged) warp.  The single-thread roles that issue TMA copies and
-// MMAs are entered through this rather than `lane == 0`, behind which the compiler has to allow for
-// several active threads, and these instructions take their operands from the warp's uniform registers.
-// Measured per instruction issued (SM cycles, one thread, the CTA's other warps waiting): tcgen05.mma with
+// MMAs are entered through this rather than `lane == 0`: it is faster.  Measured per instruction issued (SM cycles, one thread, the CTA's other warps waiting): tcgen05.mma with
 // both operands in shared memory 130 -> 65 (N <= 64: then bound by the operand reads), a 3-D TMA load
 // 47 -> 10, tcgen05.commit 49 -> 17.  Whole runs: D=2048 H=1024 T=64 B=1024 K=128 1613 -> 1398 us, K=512
 // 3060 -> 2702 us; two layers D=4096 H=2048 T=16 B=64 K=1024 with four depths 1246 -> 1119 us; D=1024 H=512
@@ -238,9 +236,9 @@ __device__ __forceinline__ float ex2_approx(float z) {
 
 constexpr float kLog2E = 1.44269504088896341f;
 
-// e^z = 2^(z log2 e) for the functions below, all of which add it to 1: a
-// result below 2^-126 may be zero, which saves the scaling around the
-// hardware instruction (three instructions of five).
+// e^z = 2^(z log2 e) for the functions below, all of which add it to 1, a sum
+// that cannot see a result below 2^-126: those may be zero (the instruction's
+// .ftz form).
 __device__ __forceinline__ float exp_for_sum(float z) { return ex2_approx(z * kLog2E); }
 
 // Logistic function 1 / (1 + e^-z) from the hardware exponential and
