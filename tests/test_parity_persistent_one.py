@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 from parity_util import FP32_TOL, assert_parity, oracle_run, run_gpu
-from paper_1905_00689_gb300 import FP32, Q_LAUNCHES, Q_PERSISTENT_VARIANT, plan
+from paper_1905_00689_gb300 import FP32, PATH_SIMT, Q_LAST_PATH, Q_LAUNCHES, Q_PERSISTENT_VARIANT, plan
 from workloads import draw_factor_set, draw_inputs
 
 
@@ -86,9 +86,19 @@ def test_lanes_past_a_row_meet_no_infinity(cuda_device, H, K, term):
     assert_parity(got, ref, FP32_TOL)
 
 
-@pytest.mark.parametrize("H,K,one", [(64, 16, 1), (64, 32, 1), (64, 33, 0), (128, 16, 1), (128, 17, 0), (129, 4, 0),
+@pytest.mark.parametrize("H,K,one", [(64, 16, 1), (64, 32, 1), (64, 33, 0), (128, 16, 1), (128, 17, 0), (132, 4, 0),
                                      (32, 64, 1), (32, 65, 0), (4, 128, 1), (4, 129, 0), (512, 16, 0)])
 def test_rule(H, K, one):
     """H, K <= 128 and at most 16 values of either factor per thread of 512."""
-    if H % 4 == 0:
-        assert plan(FP32, H, 4, 1, K)["one_cta"] == one
+    assert plan(FP32, H, 4, 1, K)["one_cta"] == one
+
+
+@pytest.mark.gpu
+def test_widths_off_the_quads_take_the_per_timestep_kernels(cuda_device):
+    """H not a multiple of 4: no persistent kernel, whatever the size."""
+    D, H, T, B, K = 20, 62, 3, 2, 6
+    gates = [draw_factor_set(H, D + H, K, 20, 9400 + g) for g in range(4)]
+    x = draw_inputs(T, B, D, "uniform", 95)
+    got, m = run_gpu([gates], x, K, checkpoints=[3])
+    assert m.query(Q_LAST_PATH) == PATH_SIMT == plan(FP32, H, T, B, K, [3])["path"]
+    assert_parity(got, oracle_run([gates], x, K, checkpoints=[3]), FP32_TOL)
