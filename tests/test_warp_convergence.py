@@ -42,12 +42,12 @@ LANE_BRANCH = re.compile(r"\b(?:e|lane|tid|threadIdx\.x) (?:==|<)|\b(?:elect_one
 def test_loads_without_a_barrier_are_reached_together(name):
     """A load that leaves the barrier out (kTogether) follows a warp-wide
     barrier or vote, or a load that has one, with no branch of single lanes
-    and no wait in between.  `load_sums` (k_tensor_loop.cu) passes the demand
-    on to its callers."""
+    and no wait in between.  `load_sums` and `read_sums` (k_tensor_loop.cu)
+    pass the demand on to their callers."""
     with open(os.path.join(CSRC, name)) as f:
         text = re.sub(r"//[^\n]*", "", f.read())
-    text = re.sub(r"auto load_sums = .*?\n    \};\n", "", text, flags=re.S)
-    for m in re.finditer(r"tmem_ld\w+<true>\(|\bload_sums\(", text):
+    text = re.sub(r"auto (?:load|read)_sums = .*?\n    \};\n", "", text, flags=re.S)
+    for m in re.finditer(r"tmem_ld\w+<true>\(|\b(?:load|read)_sums\(", text):
         last = [k for k in re.finditer(r"__syncwarp\(\);|__all_sync\(.*?\);|tmem_ld\w+\(.*?\);", text[:m.start()], re.S)][-1]
         between = text[last.end():m.start()]
         assert not LANE_BRANCH.search(between), (name, between)
