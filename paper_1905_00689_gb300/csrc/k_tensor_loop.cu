@@ -1158,15 +1158,35 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
       if ((long long)groups * ((ST + n - 1) / n) <= most) return n;
     return 0;
   };
-  // A CTA's epilogues take longer than the launches they save once its stream tiles are many.  Measured
-  // (recurrence us a step, this launch / two launches): 96 streams of both roles together (two layers of
-  // H = 2048, B = 64, K = 1024 with depths) 21 / 33; 128 (H = 1024, B = 1024, K = 128) 11.1 / 14.6; 192
-  // (H = 2048, B = 256, K = 200) 16.0 / 18.1, (H = 2048, B = 180, K = 512) 16.7 / 18.3, (H = 1024, B = 300, K = 512)
-  // 16.7 / 17.1; 256 (H = 1024, B = 600, K = 200) 22.8 / 15.8.  With several segments of terms 160 (H = 1024,
-  // B = 256, K = 640) 18.1 / 23.4; 192 (K = 1000) 33.9 / 25.8.  Up to K = 320 and H = 1024 without depths the two
-  // launches are at their best: 192 (H = 1024, B = 512, K = 200) 16.7 / 13.6, 160 (H = 512, B = 600, K = 256)
-  // 14.1 / 12.9, 96 (H = 512, B = 400, K = 200) 10.0 / 17.4.
-  const int limit = K > 512 ? 160 : p.gp == 1 && K <= 320 && H <= 1024 && p.ndep == 0 ? 128 : 192;
+  // Tiles of 16 streams spread a few streams over more CTAs and have half the sums to read and exchange per
+  // item; with many tiles per CTA those of 32 pay each item's latencies less often.  Recurrence, us a step, tiles
+  // of 16 / 32 by the stream tiles of 16 per CTA (both roles; one gate per CTA, no depths unless said): 2 (H = 512,
+  // B = 64, K = 512) 7.5 / 8.7, (K = 128, all gates) 8.0 / 9.0, (K = 512, two depths, B = 128) 9.2 / 10.9; 3 (H =
+  // 512, B = 128, K = 902) 11.6 / 13.3, (H = 1024, B = 64, K = 700, a depth) 12.3 / 13.1; 4 (H = 2048, B = 64,
+  // K = 512) 9.5 / 10.5, (H = 512, B = 1024, K = 128, all gates) 9.9 / 9.2, (H = 512, B = 256, K = 512, two depths)
+  // 12.1 / 11.4; 5 (H = 512, B = 300, K = 200) 10.9 / 10.0; 8 (H = 512, B = 512, K = 512) 15.0 / 11.4.
+  const int few = p.gp == 1 && p.ndep == 0 ? 4 : 3;
+  const int sa16 = per_cta(16, p.RT * p.ga), sb16 = per_cta(16, p.UT * gb);
+  const int first = sa16 > 0 && sb16 > 0 && sa16 + sb16 <= few ? 16 : 32;
+  // A CTA's epilogues take longer than the launches they save once its streams (of both roles together) are many.
+  // Measured, this launch / two launches, us a step: 96 streams (two layers of H = 2048, B = 64, K = 1024 with
+  // depths) 21 / 33; 128 (H = 1024, B = 1024, K = 128) 11.1 / 14.6; 192 (H = 2048, B = 256, K = 200) 17.1 / 18.9,
+  // (H = 2048, B = 180, K = 512) 17.6 / 18.6; 256 (H = 1024, B = 600, K = 200) 22.8 / 15.8.  Where the two launches
+  // are at their best, and with several segments of terms, the line lies lower (us a run of 12 steps, D = 64):
+  // - one gate per CTA, H <= 1024, no depths: 128 up to K = 448 (H > 512) or 384.  H = 1024, 160 streams (B = 300):
+  //   K = 320 203 / 177, 384 207 / 186, 448 214 / 207, 512 217 / 216; 128 (B = 256): K = 320 149 / 243.  H = 512,
+  //   160 (B = 600): K = 256 186 / 169, 384 198 / 198, 448 197 / 235; 128 (B = 500): K = 256 133 / 235.
+  // - K > 512: 160.  H = 1024, K = 640, B = 256 247 / 298; H = 512, K = 800, B = 400 291 / 345; H = 2048, K = 800,
+  //   B = 96 265 / 290; 192 (H = 2048, K = 800, B = 128) 305 / 319; but with H over two CTAs and K > 704, no
+  //   depths, 128: H = 1024, K = 800, 160 (B = 160) 293 / 267, 96 (B = 128) 199 / 228.
+  // - tiles of 16 in place of 32 for want of room: 128 with depths, else 64.  H = 2048, K = 1000, two depths, 96
+  //   (B = 64) 306 / 364, 144 (B = 96) 429 / 406; H = 1024, K = 1000, no depths, 80 (B = 96) 240 / 235, 96 251 / 230.
+  int limit = 192;
+  if (K > 512)
+    limit = p.ga == 2 && K > 704 && p.ndep == 0 ? 128 : 160;
+  else if (p.gp == 1 && p.ga <= 2 && p.ndep == 0 && K <= (p.ga == 2 ? 448 : 384))
+    limit = 128;
+  const int limit16 = first == 16 ? limit : p.ndep > 0 ? 128 : 64;
   // fills in the tile width nt with ures 64-term chunks of U in tensor memory; false if it does not fit
   auto fit = [&](int nt, int ures, TcLoopPlan* o) {
     TcLoopPlan c = p;
@@ -1176,7 +1196,7 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     if (c.ST > kLoopMaxTiles) return false;
     c.sa = per_cta(nt, c.RT * c.ga);
     c.sb = per_cta(nt, c.UT * gb);
-    if (c.sa == 0 || c.sb == 0 || (c.sa + c.sb) * nt > limit) return false;
+    if (c.sa == 0 || c.sb == 0 || (c.sa + c.sb) * nt > (nt == 16 ? limit16 : limit)) return false;
     c.nA = c.RT * c.ga * ((c.ST + c.sa - 1) / c.sa);
     c.nB = c.UT * gb * ((c.ST + c.sb - 1) / c.sb);
     const int n = c.nA > c.nB ? c.nA : c.nB;
@@ -1223,19 +1243,9 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
     *o = c;
     return true;
   };
-  // Tiles of 16 streams spread a few streams over more CTAs and have half the sums to read and exchange per
-  // item; with many tiles per CTA those of 32 pay each item's latencies less often.  Recurrence, us a step, tiles
-  // of 16 / 32 by the stream tiles of 16 per CTA (both roles; one gate per CTA, no depths unless said): 2 (H = 512,
-  // B = 64, K = 512) 7.5 / 8.7, (K = 128, all gates) 8.0 / 9.0, (K = 512, two depths, B = 128) 9.2 / 10.9; 3 (H =
-  // 512, B = 128, K = 902) 11.6 / 13.3, (H = 1024, B = 64, K = 700, a depth) 12.3 / 13.1; 4 (H = 2048, B = 64,
-  // K = 512) 9.5 / 10.5, (H = 512, B = 1024, K = 128, all gates) 9.9 / 9.2, (H = 512, B = 256, K = 512, two depths)
-  // 12.1 / 11.4; 5 (H = 512, B = 300, K = 200) 10.9 / 10.0; 8 (H = 512, B = 512, K = 512) 15.0 / 11.4.
   // Among the ways to hold U: separate accumulators for the two roles first, then as much of U as possible in
   // tensor memory.
   TcLoopPlan c;
-  const int few = p.gp == 1 && p.ndep == 0 ? 4 : 3;
-  const int sa16 = per_cta(16, p.RT * p.ga), sb16 = per_cta(16, p.UT * gb);
-  const int first = sa16 > 0 && sb16 > 0 && sa16 + sb16 <= few ? 16 : 32;
   // (tiles of 16 in place of 32 for want of room do not make more streams fit)
   if (first == 32 && (per_cta(32, p.RT * p.ga) + per_cta(32, p.UT * gb)) * 32 > limit) return false;
   for (int nt : {first, 48 - first})

@@ -217,3 +217,15 @@ def test_rule(H, B, K, cps, loop):
     p = plan(BF16, H, 2, B, K, cps)
     assert p["tensor_loop"] == loop
     assert p["tensor_seq"] == (1 if K <= 32 and H == 512 else 0)
+
+
+@pytest.mark.parametrize("H,B,K,cps,loop", [
+    (1024, 256, 448, [], 1), (1024, 300, 448, [], 0), (1024, 300, 512, [], 1),    # 128, 160, 160 streams per CTA
+    (512, 500, 384, [], 1), (512, 600, 384, [], 0), (512, 600, 448, [], 1),
+    (1024, 128, 800, [], 1), (1024, 160, 800, [], 0), (512, 400, 800, [], 1),
+    (1024, 64, 1000, [], 1), (1024, 96, 1000, [], 0),                             # tiles of 16 for want of room
+    (2048, 64, 1000, [64, 320], 1), (2048, 96, 1000, [64, 320], 0),
+])
+def test_limits(H, B, K, cps, loop):
+    """Either side of the measured lines between this launch and two launches per step."""
+    assert plan(BF16, H, 12, B, K, cps)["tensor_loop"] == loop
