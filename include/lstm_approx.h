@@ -310,8 +310,9 @@ enum lstm_approx_option_key {
                                intermediate depths multiples of 16 or >= K,
                                masked-dense tau'; else one launch over all
                                tiles for all T where the factors and the
-                               streams fit the GPU's CTAs: H <= 2048,
-                               K <= 1024), 1 = two launches per timestep.
+                               streams fit the GPU's CTAs, H <= 2048,
+                               K <= 1024, and the timesteps are enough to
+                               pay for loading them), 1 = two launches per timestep.
                                The launch over all tiles is cooperative: its
                                up to 148 CTAs start together, once the other
                                kernels on the GPU have left that many SMs,

@@ -274,6 +274,41 @@ TensorTiles tensor_tiles(int H, int B, int K, const Checkpoints& ck) {
   return t;
 }
 
+// Whether a run of T timesteps takes the resident-factor launch where its plan fits.  It loads the factors into
+// tensor and shared memory before its first step and needs its whole grid at once, 8 to 18 us more than the launches
+// per step take to start, and gains 2 to 30 us a step: with few timesteps it can lose (us a call, this launch / launches
+// per step: H = 256, B = 64, K = 1000 T = 1 39.5 / 24.9, T = 4 69 / 65; H = 136, B = 40, K = 48 T = 1 24.0 / 18.8,
+// T = 2 28.5 / 26.7, T = 4 38.9 / 42.9; but H = 1024, B = 256, K = 200 T = 1 30.7 / 37.3; H = 600, B = 100, K = 90 with
+// two depths T = 1 34.6 / 38.9).  The times below are fits to 299 shapes at T = 1, 2, 3, 4 and 6, within about 2 us: a
+// term for each thing a CTA does in turn.  By them the way that is slower by more than 10% is taken in 15 of those
+// 1495 runs (always this launch: in 184), and in 12 (116) of 935 runs of 187 other shapes.  Beyond one step and with
+// more than 96 streams per CTA the plan's own limits decide.
+bool loop_pays(const TcLoopPlan& p, const TensorTiles& t, int H, int B, int K, int T, const Checkpoints& ck) {
+  if (T > 8 || (T > 1 && (p.sa + p.sb) * p.nt > 96)) return true;
+  auto div_up = [](int a, int b) { return (a + b - 1) / b; };
+  const int chunks = div_up(K, 64), slices = div_up(K, 16), J = ck.n;
+  // resident-factor launch: slices of U written to tensor memory, chunks beside them, streams and terms per step
+  int pieces = slices < 4 * p.ures ? slices : 4 * p.ures;
+  for (int j = 0; j < p.ndep; ++j) pieces += ck.k[j] % 16 != 0 ? 1 : 0;
+  const float split_h = p.ga > 1 ? 1.f : 0.f, one_gate = p.gp == 1 ? 1.f : 0.f;
+  const float loop_set_up = 14.8f + 0.29f * (pieces * p.gp) + 0.6f * (chunks - p.ures) + 0.7f * split_h + 1.2f * one_gate +
+                            1.0f * p.ndep;
+  const float loop_step = 2.6f + 0.005f * K + 0.078f * ((p.sa + p.sb) * p.nt) + 1.1f * split_h - 1.2f * one_gate +
+                          0.75f * p.ndep;
+  // launches per step: waves of tau' and gate tiles, 64-element chunks per tile, columns per tile, the reduce kernel
+  const int row_tiles = tensor_rows_per_gate(K) > 0 ? 1 : 4 * div_up(K, 128);
+  const int waves_a = div_up(row_tiles * div_up(B, t.bnh) * t.sk, 148);
+  const int waves_b = div_up(div_up(H, 128) * div_up(B, t.nt) * t.ks, 148);
+  int odd = 0;  // depths off the 16-term slices
+  for (int j = 0; j < J; ++j) odd += ck.k[j] % 16 != 0 ? 1 : 0;
+  const float cells = 1e-6f * H * B;
+  const float step = -1.8f + waves_a * (0.15f * div_up(div_up(H, 64), t.sk) + 0.157f * t.bnh) +
+                     waves_b * (1.23f * div_up(chunks, t.ks) + 0.077f * t.nt) + 2.0f * J + 2.7f * odd +
+                     23.f * J * cells + (t.raw ? 3.4f + 8.9f * t.ks * cells : 0.f);
+  const float steps_set_up = 12.5f + 4.6f * cells;
+  return 0.97f * (loop_set_up + T * loop_step) <= steps_set_up + T * step;
+}
+
 // The compressed h part of layer l's v on the device, for the compressed
 // tau' layout: CSR over the storage rows g*Ks + k of all four gates (rows not
 // set: empty), assembled from the per-gate host copies that set_factors
@@ -446,7 +481,9 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
   }
   h->last_tensor_seq = 0;
   TcLoopPlan lp;
-  if (h->opt_tensor_seq == 0 && h->opt_tau_layout == 0 && tc_loop_plan(H, B, K, ck, &lp)) {
+  const TensorTiles tt = tensor_tiles(H, B, K, ck);
+  if (h->opt_tensor_seq == 0 && h->opt_tau_layout == 0 && tc_loop_plan(H, B, K, ck, &lp) &&
+      loop_pays(lp, tt, H, B, K, T, ck)) {
     // one launch over all stream tiles for all T timesteps, the factors resident (offsets within a
     // timestep's P are 32-bit there: B * ldp below 2^31 follows from its limits on B and K)
     TcMap mh, mt;
@@ -506,7 +543,6 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
   // gate GEMM reads 64-term chunks, so the rest of the pair must be zero
   if (rpg > 0)
     LA_CUDA(h, cudaMemsetAsync(tau, 0, 2ull * B * 4 * h->Ks * sizeof(__nv_bfloat16), h->stream), "tau' clear");
-  const TensorTiles tt = tensor_tiles(H, B, K, ck);
   const int bnh = tt.bnh, nt = tt.nt, ks = tt.ks, nkb_per = tt.nkb_per;
   if (tt.raw) {
     const size_t need = (size_t)(ks + ck.n) * 4 * B * H * sizeof(float);
@@ -1403,7 +1439,8 @@ int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int* chec
       v[LSTM_APPROX_PLAN_GATE_SPLITS] = tt.ks;
       v[LSTM_APPROX_PLAN_TAU_SPLITS] = tt.sk;
       TcLoopPlan lp;
-      v[LSTM_APPROX_PLAN_TENSOR_LOOP] = tc_loop_plan(hidden, B, K, ck, &lp) ? 1 : 0;
+      v[LSTM_APPROX_PLAN_TENSOR_LOOP] =
+          tc_loop_plan(hidden, B, K, ck, &lp) && loop_pays(lp, tt, hidden, B, K, T, ck) ? 1 : 0;
     }
   }
   for (int i = 0; i < n_out; ++i) out[i] = i < LSTM_APPROX_PLAN_ITEMS ? v[i] : 0;

@@ -148,8 +148,8 @@ def test_bounded_wait_reports_timeout(cuda_device, H, K):
 @pytest.mark.parametrize("H,B,K,cps", [
     (136, 40, 40, [10, 32]),    # all gates in a CTA
     (512, 70, 200, [64, 100]),  # one gate per CTA
-    (512, 40, 902, [451]),      # segments
-    (1024, 300, 128, [64]),     # several stream tiles per CTA
+    (512, 256, 640, [320]),     # segments
+    (512, 1000, 100, [50]),     # several stream tiles per CTA
 ])
 def test_state_in_place(cuda_device, H, B, K, cps, T):
     """The same buffers as initial and final state (a caller that resumes one
@@ -229,3 +229,29 @@ def test_rule(H, B, K, cps, loop):
 def test_limits(H, B, K, cps, loop):
     """Either side of the measured lines between this launch and two launches per step."""
     assert plan(BF16, H, 12, B, K, cps)["tensor_loop"] == loop
+
+
+@pytest.mark.parametrize("H,B,K,cps,T,loop", [
+    (256, 64, 1000, [], 1, 0), (256, 64, 1000, [], 2, 0), (256, 64, 1000, [], 9, 1),
+    (136, 40, 48, [], 1, 0), (136, 40, 48, [], 4, 1),
+    (1024, 256, 200, [], 1, 1), (600, 100, 90, [10, 45], 1, 1),
+    (1024, 1024, 128, [], 1, 0), (1024, 1024, 128, [], 2, 1),      # many streams: from two steps on
+])
+def test_few_timesteps(H, B, K, cps, T, loop):
+    """A run too short to pay for loading the factors takes the launches per step."""
+    assert plan(BF16, H, T, B, K, cps)["tensor_loop"] == loop
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,B,K,cps", [(256, 64, 1000, []), (136, 40, 48, [10]), (512, 33, 129, [128])])
+def test_few_timesteps_run_what_the_plan_says(cuda_device, H, B, K, cps):
+    D = 40
+    gates = _gates(H, D + H, K, 60, 8800 + H)
+    for T in (1, 2, 9):
+        x = draw_inputs(T, B, D, "uniform", 88)
+        got, m = run_gpu([gates], x, K, dtype="bf16", checkpoints=cps)
+        assert m.query(Q_TENSOR_LOOP) == plan(BF16, H, T, B, K, cps)["tensor_loop"]
+        streams = sorted({0, B // 2, B - 1})
+        ref = oracle_run([gates], x[:, streams], K, dtype="bf16", checkpoints=cps)
+        cut = {k: v[:, streams] if k in ("h", "c_last") else v[:, :, streams] for k, v in got.items()}
+        assert_parity(cut, ref, BF16_TOL)
