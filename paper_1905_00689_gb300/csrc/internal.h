@@ -335,6 +335,9 @@ struct TcRowsArgs {
 };
 // `bn` (64, 128 or 256) must match the box rows of Bm's map.
 cudaError_t launch_tc_rows(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, int n_cols, int bn, cudaStream_t s);
+// Whether the projection over n_cols columns (128-column tiles) is faster converting x inside, two row tiles per
+// CTA, than with a conversion pass before it.
+bool tc_rows_converts(int n_cols, int row_tiles, int Kdim);
 // The projection (mode 0) from fp32 activations: Xf maps the fp32 [N][Kdim]
 // input in boxes of 32 columns x 64 rows (packed gates) or x 128 rows
 // (tc_make_map_f32), and the kernel forms the bf16 pair itself.

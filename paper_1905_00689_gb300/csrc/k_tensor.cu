@@ -1049,6 +1049,36 @@ int tc_gates_tile_n(int H, int B) {
   return 128;
 }
 
+// The projection over many columns (128-column tiles, one CTA per SM): two row tiles per CTA move 64 KB per 64 terms for
+// the work of two, but a CTA takes 0.78 us per 64 terms (0.92 if it converts x as well) where one with one row tile takes
+// 0.445, and the grid has half the CTAs.  So what counts is waves: one wave either way, or three against two, is for one
+// tile.  Measured (a layer of H = 128, us, one tile and the conversion pass / two tiles converting inside / two tiles
+// and the pass): D = 4096, K = 64, T B = 2400 72 / 84 / 89 (one wave each), 8000 158 / 119 / 147 (2 and 1); K = 512,
+// T B = 2800 148 / 167 / 158 (3 and 2), 4000 189 / 177 / 174 (4 and 2); D = 1024, K = 64, 2400 49 / 53 / 55.
+namespace {
+constexpr int kSms = 152;
+struct RowWaves {
+  int one, two;
+};
+RowWaves rows_waves(int n_cols, int row_tiles) {
+  const int col_tiles = (n_cols + 127) / 128;
+  return {(row_tiles * col_tiles + kSms - 1) / kSms, (row_tiles / 2 * col_tiles + kSms - 1) / kSms};
+}
+bool rows_two_tiles(int n_cols, int row_tiles) {
+  const RowWaves w = rows_waves(n_cols, row_tiles);
+  return 10 * w.one > 16 * w.two;
+}
+}  // namespace
+
+bool tc_rows_converts(int n_cols, int row_tiles, int Kdim) {
+  const RowWaves w = rows_waves(n_cols, row_tiles);
+  const float chunks = (float)((Kdim + 63) / 64);
+  // the pass: its launch, x read and its pair written
+  const float pass = 2.5f + 1.3e-6f * n_cols * Kdim;
+  const float from_pair = rows_two_tiles(n_cols, row_tiles) ? 0.78f * w.two : 0.445f * w.one;
+  return 0.92f * w.two * chunks <= pass + from_pair * chunks;
+}
+
 cudaError_t launch_tc_rows_xf32(const TcMap& A, const TcMap& Xf, const TcRowsArgs& a, int n_cols, cudaStream_t s) {
   return a.rpg > 0 ? launch_rows_t<64, 6, true>(A, Xf, a, n_cols, s)
                    : launch_rows_t<128, 3, true, 2>(A, Xf, a, n_cols, s);
@@ -1089,8 +1119,9 @@ bool tc_make_map_planes(TcMap* m, const void* base, uint64_t inner, uint64_t row
 cudaError_t launch_tc_rows(const TcMap& A, const TcMap& Bm, const TcRowsArgs& a, int n_cols, int bn, cudaStream_t s) {
   switch (bn) {
     case 128:
-      return a.mode == 0 && a.rpg == 0 ? launch_rows_t<128, 3, false, 2>(A, Bm, a, n_cols, s)
-                                       : launch_rows_t<128, 4>(A, Bm, a, n_cols, s);
+      return a.mode == 0 && a.rpg == 0 && rows_two_tiles(n_cols, 4 * a.kt_per_gate)
+                 ? launch_rows_t<128, 3, false, 2>(A, Bm, a, n_cols, s)
+                 : launch_rows_t<128, 4>(A, Bm, a, n_cols, s);
     case 32: return launch_rows_t<32, 8>(A, Bm, a, n_cols, s);
     default: return launch_rows_t<64, 6>(A, Bm, a, n_cols, s);
   }

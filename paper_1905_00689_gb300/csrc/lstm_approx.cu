@@ -397,10 +397,10 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
   // (one tile of rows, x converted once) and over many columns (two row tiles per CTA, each pair of row tiles
   // converting it again beside its MMAs; the separate pass reads x and writes its pair, the same bytes again).
   // D=2048, T B=65536, conversion and projection: K=128 402 -> 239 us, K=512 978 -> 851; at K = 1024, D = 4096, T B =
-  // 1024 the pass and the projection from the pair are as fast.
+  // 1024 the pass and the projection from the pair are as fast, and with few waves of CTAs faster (tc_rows_converts).
   const int bnx = tc_rows_tile_n(TB, rpg > 0 ? 1 : 4 * ((K + 127) / 128));
   const bool x_f32 =
-      l == 0 && (rpg > 0 || (bnx == 128 && K <= 512)) && D % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
+      l == 0 && (rpg > 0 || (bnx == 128 && K <= 512 && tc_rows_converts(TB, 4 * ((K + 127) / 128), D))) && D % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
   if (l == 0 && !x_f32) {  // operand conversion (outside the timed projection phase)
     LA_CUDA(h, launch_to_bf16(x, TB, D, static_cast<__nv_bfloat16*>(h->x_bf16), s.ldx, h->stream),
             "input conversion launch");

@@ -10,6 +10,27 @@ from workloads import draw_factor_set, draw_inputs
 pytestmark = pytest.mark.gpu
 
 
+def _check(D, T, B, K, layers, H=64):
+    lay = [[draw_factor_set(H, (D if l == 0 else H) + H, K, 30, 9700 + 10 * l + g) for g in range(4)]
+           for l in range(layers)]
+    x = draw_inputs(T, B, D, "uniform", 97)
+    got, m = run_gpu(lay, x, K, dtype="bf16", checkpoints=[K // 2])
+    streams = [0, 63, B - 1]
+    ref = oracle_run(lay, x[:, streams], K, dtype="bf16", checkpoints=[K // 2])
+    cut = {k: v[:, streams] if k in ("h", "c_last") else v[:, :, streams] for k, v in got.items()}
+    assert_parity(cut, ref, BF16_TOL)
+
+
+@pytest.mark.parametrize("D,T,B,K", [
+    (2052, 8, 300, 40),    # one wave either way: one row tile per CTA, x converted by a pass
+    (2050, 8, 303, 128),   # the same with rows of x TMA cannot map
+    (1024, 8, 350, 512),   # three waves against two
+    (65, 66, 97, 300),     # five against three: two row tiles, an odd number per gate, from the pair
+])
+def test_tiles_by_waves(cuda_device, D, T, B, K):
+    _check(D, T, B, K, layers=2)
+
+
 @pytest.mark.parametrize("D,T,B,K", [
     (72, 40, 130, 40),     # one row tile per gate (a CTA's two tiles are two gates), ragged columns, D off the 64s
     (42, 40, 130, 40),     # rows of x TMA cannot map: converted by a pass before
