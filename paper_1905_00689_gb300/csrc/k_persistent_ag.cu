@@ -617,8 +617,14 @@ bool choose_persistent(int H, int K, int T, int B, const Checkpoints& ck, int wa
   // More streams than resident clusters: a second wave takes as long as the first, so a smaller cluster that
   // holds them all is faster although its step is longer.  20 steps at H = 512, K = 64: 8 streams 73.2 us on
   // clusters of 16, 40.4 on 8; 24 streams 140.8, 77.2, 50.7 (one-exchange kernel on 4); H = 256, K = 200, 8
-  // streams 85.5 (one-exchange, 16), 67.1 (8).  Relative time of a step by kernel and cluster size:
-  auto weight = [](int v, int cs) { return v == 1 ? (cs == 16 ? 10 : cs == 8 ? 11 : 13) : (cs == 8 ? 11 : 12); };
+  // streams 85.5 (one-exchange, 16), 67.1 (8).  Relative time of a step by kernel and cluster size; with more than 64
+  // terms the per-unit-block kernel in place of the one-exchange kernel on the next larger cluster takes 1.5 to 1.8
+  // times as long (H = 256, K = 128 72.8 us on 4 against 40.1 on 8: 37 streams 145 in two waves, 120 in three;
+  // K = 256 72.7 on 8 against 44.7 on 16: 16 streams 144, 132):
+  const bool from_ag = c->variant == 2 && K > 64;
+  auto weight = [from_ag](int v, int cs) {
+    return v == 1 ? (from_ag ? 19 : cs == 16 ? 10 : cs == 8 ? 11 : 13) : (cs == 8 ? 11 : 12);
+  };
   auto cost = [&](int v, int cs) { return (long long)((B + resident_clusters(cs) - 1) / resident_clusters(cs)) * weight(v, cs); };
   long long best = cost(c->variant, c->CS);
   for (int v : {1, 2})

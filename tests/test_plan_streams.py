@@ -20,3 +20,13 @@ def test_streams_choose_the_cluster(H, K, B, variant, cluster):
     assert (p["persistent_variant"], p["cluster"]) == (variant, cluster)
     if cluster < 16:
         assert B <= RESIDENT[cluster]
+
+
+@pytest.mark.parametrize("H,K,B,variant,cluster", [
+    (256, 128, 37, 2, 8), (256, 128, 46, 1, 4),   # three waves against two, four against two
+    (256, 256, 8, 1, 8), (256, 256, 16, 2, 16), (256, 256, 22, 1, 8),
+])
+def test_many_terms_keep_the_one_exchange_kernel(H, K, B, variant, cluster):
+    """The per-unit-block kernel on the smaller cluster takes 1.5 to 1.8 times as long."""
+    p = plan(FP32, H, 20, B, K)
+    assert (p["persistent_variant"], p["cluster"]) == (variant, cluster)
