@@ -278,7 +278,7 @@ struct OneProj {
   int ldx = 0;
   SparseXRows sparse{};
 };
-bool plan_persistent_one(int H, int K, bool gathers, PersistentOnePlan* out);  // gathers: OneProj mode 2
+bool plan_persistent_one(int H, int K, int T, const Checkpoints& ck, bool gathers, PersistentOnePlan* out);  // gathers: OneProj mode 2
 int persistent_one_projection(int K, int T, int D, long long kept_x, bool sparse);
 cudaError_t launch_persistent_one(const PersistentOnePlan& p, const PersistentArgs& a, const OneProj& pr,
                                   cudaStream_t s);

@@ -335,12 +335,12 @@ int pow2_at_most(int v) {
 
 }  // namespace
 
-bool plan_persistent_one(int H, int K, bool gathers, PersistentOnePlan* out) {
+bool plan_persistent_one(int H, int K, int T, const Checkpoints& ck, bool gathers, PersistentOnePlan* out) {
   if (H < 1 || H > 128 || K < 1 || K > 128) return false;
   // The fewest threads that hold the factors in 4 quads each; 512 where compressed rows of x are gathered (entries
   // in flight).  With 8 quads a step takes longer than the one-exchange cluster kernel's and the set-up as long:
   // T = 32, H = 64, K = 64 55.7 us against 49.7, H = 128, K = 32 57.8 / 45.6, H = 32, K = 96 60.0 / 47.7; with 4
-  // H = 64, K = 32 44.6 / 45.3, H = 32, K = 64 47.5 / 49.7, H = 64, K = 16 33.9 / 43.4.
+  // H = 64, K = 16 31.2 / 41.3, H = 32, K = 32 32.3 / 41.5 (256 threads; 512: below).
   PersistentOnePlan p;
   for (int nth = 128; nth <= kMaxThreads; nth *= 2) {
     if (4 * K > nth || 4 * H > nth || (gathers && nth < kMaxThreads)) continue;
@@ -356,6 +356,16 @@ bool plan_persistent_one(int H, int K, bool gathers, PersistentOnePlan* out) {
   }
   return false;
 found:
+  // With 512 threads of 16 values each a step without intermediate depths takes longer than the cluster kernel's
+  // (1.32 us against 1.03 at H = 64, K = 32, 1.18 at H = 128, K = 16; with a depth 1.5 / 2 or less), and only the
+  // set-up is shorter (4 us against 8.5).  Calls back to back and single calls, us, this kernel / cluster kernel:
+  // H = 64, K = 32 T = 8 13.4 / 16.7 and 28.6 / 28.5, T = 12 20.0 / 20.9 and 36.1 / 32.6, T = 20 30.8 / 29.2 and
+  // 47.4 / 40.7, T = 32 46.1 / 41.6; H = 128, K = 16 T = 20 27.3 / 29.1 and 43.4 / 40.2, T = 32 41.3 / 41.4 and 56.7 /
+  // 53.1, T = 64 80.0 / 74.3.
+  // (H = 8, K = 96 T = 32 43.3 / 45.5.)
+  if (p.threads == 512 && p.VQ == kMaxQuads && H >= 32 && !gathers && T > (K > 16 ? 12 : 20) &&
+      (ck.n == 0 || ck.k[0] >= K))
+    return false;
   p.HP = (H + 3) / 4 * 4 + 4;
   // the four gates' rows eight banks apart, so that the 16-byte reads of a unit's lanes do not collide
   p.KP = ((K + 3) / 4 * 4 + 4 + 23) / 32 * 32 + 8;

@@ -722,7 +722,7 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
     PersistentOnePlan one;
     const bool use_one = path == LSTM_APPROX_PATH_PERSISTENT && h->opt_force_path == 0 && h->opt_cluster == 0 &&
                          h->opt_persistent_variant == 0 && h->opt_xproj == 0 && h->opt_test_stall == 0 &&
-                         plan_persistent_one(H, K, false, &one);
+                         plan_persistent_one(H, K, T, lck, false, &one);
     OneProj one_proj;
     if (use_one && B <= kOneProjMaxStreams) {  // every CTA reads the projection's rows: not for many streams
       long long kept = 0;
@@ -742,7 +742,7 @@ int run_device(lstm_approx_t* h, const float* x, int T, int B, int K, const floa
         one_proj.sparse.idx[g] = s.xidx[g];
         one_proj.sparse.val[g] = s.xval[g];
       }
-      if (one_proj.mode == 2 && !plan_persistent_one(H, K, true, &one)) one_proj.mode = 0;
+      if (one_proj.mode == 2 && !plan_persistent_one(H, K, T, lck, true, &one)) one_proj.mode = 0;
     }
     const bool sparse_x = sparse_x_projection(h, s, K, T * B);
     const bool cluster_x = !sparse_x && xproj_cluster_fits(T * B, s.D, s.Vx, s.ldx, in, s.D, bf16);
@@ -1422,7 +1422,7 @@ int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int* chec
       v[LSTM_APPROX_PLAN_TMEM_COLUMNS] = pc.ag.tcols;
     }
     PersistentOnePlan one;
-    v[LSTM_APPROX_PLAN_ONE_CTA] = plan_persistent_one(hidden, K, false, &one) ? 1 : 0;
+    v[LSTM_APPROX_PLAN_ONE_CTA] = plan_persistent_one(hidden, K, T, ck, false, &one) ? 1 : 0;
   } else if (path == LSTM_APPROX_PATH_TENSOR) {
     int ns = 0, mt = 0;
     if (tc_seq_fits(hidden, B, K, ck, &ns, &mt, nullptr)) {

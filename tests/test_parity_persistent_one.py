@@ -102,3 +102,22 @@ def test_widths_off_the_quads_take_the_per_timestep_kernels(cuda_device):
     got, m = run_gpu([gates], x, K, checkpoints=[3])
     assert m.query(Q_LAST_PATH) == PATH_SIMT == plan(FP32, H, T, B, K, [3])["path"]
     assert_parity(got, oracle_run([gates], x, K, checkpoints=[3]), FP32_TOL)
+
+
+@pytest.mark.parametrize("H,K,T,cps,one", [
+    (64, 32, 12, [], 1), (64, 32, 13, [], 0), (64, 32, 13, [8], 1), (64, 32, 13, [32], 0),
+    (128, 16, 20, [], 1), (128, 16, 21, [], 0), (64, 16, 100, [], 1), (128, 8, 100, [], 1), (8, 96, 32, [], 1),
+])
+def test_rule_for_many_timesteps(H, K, T, cps, one):
+    """512 threads of 16 values: a longer step than the cluster kernel's without depths below K."""
+    assert plan(FP32, H, T, 1, K, cps)["one_cta"] == one
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,K,T,variant", [(64, 32, 12, 3), (64, 32, 13, 2), (128, 16, 21, 2)])
+def test_many_timesteps_run_what_the_plan_says(cuda_device, H, K, T, variant):
+    gates = [draw_factor_set(H, 24 + H, K, 40, 9380 + g) for g in range(4)]
+    x = draw_inputs(T, 2, 24, "uniform", 96)
+    got, m = run_gpu([gates], x, K)
+    assert m.query(Q_PERSISTENT_VARIANT) == variant
+    assert_parity(got, oracle_run([gates], x, K), FP32_TOL)
