@@ -141,13 +141,6 @@ __device__ __forceinline__ void bulk_copy_s2cluster(uint32_t dst_cluster, uint32
       : "memory");
 }
 
-// 4-byte load from shared memory of a CTA of the cluster (address from mapa).
-__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-
 // Orders this thread's generic-proxy shared-memory writes before later
 // async-proxy (bulk copy) reads of them.
 __device__ __forceinline__ void fence_proxy_async_shared() {
@@ -207,17 +200,6 @@ __device__ __forceinline__ bool wait_flags_epoch(const unsigned* flags, int n, u
     else if (now - t0 > limit_ns) return false;
     __nanosleep(32);
   }
-}
-
-// Makes a value opaque to the compiler, so that it stays in its register for
-// the rest of a persistent kernel instead of being loaded again from memory
-// where it is used.
-__device__ __forceinline__ void keep_in_register(float& v) { asm volatile("" : "+f"(v)); }
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 
 // 1/x from the hardware approximation (rcp.approx: about 1 ulp; 1/inf = 0).
@@ -549,13 +531,6 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
   d |= static_cast<uint64_t>(1) << 46;                   // descriptor version of tcgen05
   d |= static_cast<uint64_t>(2) << 61;                   // 128-byte swizzle
   return d;
-}
-
-// The same with 8-row groups `sbo` bytes apart (a multiple of 1024), for a
-// tile whose row groups are interleaved with other tiles' groups.
-__device__ __forceinline__ uint64_t umma_desc_sw128_sbo(uint32_t saddr, uint32_t sbo) {
-  return (umma_desc_sw128(saddr) & ~(static_cast<uint64_t>(0x3FFF) << 32)) |
-         (static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32);
 }
 
 // Byte offset of bf16 element k (< 64) of row r in a K-major tile of
