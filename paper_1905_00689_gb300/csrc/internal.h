@@ -414,7 +414,7 @@ struct TcSeqArgs {
   int test_stall;           // 1: CTA 0 of the first tile withholds its first partial tau' (the waits run out)
 };
 // Whether a layer of this shape takes the one-launch kernel; *ns receives
-// its streams per tile (32 or 64), *mt its 128-unit tiles per CTA (1 or 2).
+// its streams per cluster (16, 32 as two chains of 16, or 64), *mt its 128-unit tiles per CTA (1 or 2).
 bool tc_seq_fits(int H, int B, int K, const Checkpoints& ck, int* ns, int* mt, std::string* why);
 // Vh_p: the packed V_h map with boxes of rpg rows; U64: U as 32-term boxes of
 // 128 rows with 64-byte swizzling.

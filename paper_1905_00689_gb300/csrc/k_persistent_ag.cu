@@ -455,8 +455,9 @@ __global__ void __launch_bounds__(kThreads, 1) persistent_ag_kernel(PersistentAr
 }  // namespace
 
 namespace {
-// Clusters of cs CTAs (one per SM) resident at once on a GB300: measured by the streams at which a second
-// wave starts.
+// Clusters of cs CTAs (one per SM) resident at once on a GB300's 152 SMs: measured by the streams at which a second
+// wave starts.  They choose among kernels with the same results; where fewer fit (part of a GPU) the choice can be the
+// slower one.
 int resident_clusters(int cs) { return cs == 16 ? 7 : cs == 8 ? 15 : cs == 4 ? 36 : cs == 2 ? 76 : 152; }
 }  // namespace
 
@@ -502,8 +503,10 @@ bool plan_persistent_ag(int H, int K, int B, const Checkpoints& ck, int want_cs,
     plan->hq = hq;
     plan->smem = smem;
     // the smallest cluster that fits moves the fewest partials, except that 48 or more terms per CTA take
-    // longer than the next size's extra partials (recurrence of 20 steps, clusters of 4 / 8: H = 200, K = 50
-    // 38.4 / 34.3 us, H = 256, K = 64 38.4 / 36.4; with 16 terms per CTA, H = 512, K = 16, 36.4 / 40.4)
+    // longer than the next size's extra partials (20 steps, clusters of 4 / 8: H = 128, K = 48 31.7 / 31.4 us, K = 52
+    // 33.7 / 31.4, H = 200, K = 48 35.8 / 33.8, K = 52 37.7 / 33.7, H = 256, K = 48 35.9 / 35.6, K = 64 37.9 / 35.5;
+    // with 16 terms per CTA, H = 512, K = 16, 37.6 / 41.8).  Below H = 128 the gain at these K is as large (H = 96,
+    // K = 52 33.6 / 29.7) and not taken; above H = 256 the per-unit-block kernel or clusters of 4 serve.
     PersistentAgPlan wider;
     std::string unused;
     if (want_cs == 0 && cs == 4 && p.RA >= 48 && H >= 128 && H <= 256 && B <= resident_clusters(8) &&

@@ -25,7 +25,8 @@
 // activation with TMA (128-byte swizzle) through an S-stage mbarrier ring,
 // one thread of warp 1 issues tcgen05.mma (M = 128, N = 2 BN, K = 16 per
 // instruction) into a tensor-memory accumulator, and warps
-// 4..11 (two per 32-lane quarter of tensor memory) read it back with
+// 4..11 (two per 32-lane quarter of tensor memory; 4..19 where they convert x
+// for two row tiles) read it back with
 // tcgen05.ld for the epilogue: store P, or form tau' and store it as its
 // bf16 pair.  For tau' the epilogue warps load their P_t values into
 // registers while the mainloop streams.
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(rows_threads(XF, MT), 1)
     umma_commit(accum_bar);
     umma_commit(drain_bar);
     wait_cta(drain_bar, 0, limit, err);
-  } else if (warp >= 4) {  // ---- epilogue: warps 4..11, two per lane quarter ----
+  } else if (warp >= 4) {  // ---- epilogue: kEw warps from warp 4 on, two or four per lane quarter ----
     const int ep = warp - 4, q = ep & 3;
     constexpr int kHalf = BN / (kEw / 4);  // columns per epilogue warp
     if constexpr (XF) {  // each stage's fp32 activation tile -> its bf16 pair, in place

@@ -13,7 +13,7 @@
 //     8, 16 or 32 >= K, the A operand of the tau' product), 32 KB per 128 units;
 //   - its rows of U, the first 32 terms of each gate, 32 KB per 128 units;
 //   - h_{t-1} of its units as the bf16 pair (the B operand of the tau'
-//     product), c_{t-1} in registers of the epilogue threads;
+//     product), and c_{t-1} (each epilogue thread its own cells) in shared memory;
 //   - tau' of all terms and the tile's streams as the bf16 pair (the B
 //     operand of the gate product).
 //
@@ -22,11 +22,12 @@
 //        sum_{j in CTA} Vh[(g,k)][j] h_{t-1}[n][j]  (M = 128, N = NS);
 //   exchange 1: the epilogue warps read the partials from tensor memory and
 //        send each CTA the columns of the streams it owns (SP = NS / CS
-//        streams per CTA, 8 or 16) with st.async;
+//        streams per CTA, 4, 8 or 16) with st.async;
 //   the owner adds the CS partials in rank order, forms
 //        tau' = sigma (sum + P_t) (zero for k >= K) and its pair, writes them
 //        into its tau' operand and, exchange 2, copies that block to every
-//        other CTA with one bulk copy each;
+//        other CTA by bulk copies (one, or eight where SP = 4 is half a
+//        stream group);
 //   (a3, a6) the four gate sums of the CTA's units, y_g = U_g tau'_g (one
 //        tensor-memory accumulator per gate and 128 units), cut at each
 //        intermediate depth (a multiple of 16) for the checkpoint cells, as
@@ -615,10 +616,10 @@ bool tc_seq_fits(int H, int B, int K, const Checkpoints& ck, int* ns, int* mt, s
   if (K > 32) return no("K above 32 (the factors of a CTA's units would not fit in shared memory)");
   for (int j = 0; j < ck.n; ++j)
     if (ck.k[j] % 16 != 0 && ck.k[j] < K) return no("an intermediate depth off the 16-term slices");
-  // the narrowest tiles (16, 32 streams) whose clusters of 4 (or 2) CTAs fit
-  // in one wave; each CTA owns 4, 8 or 16 streams of a tile, so its tau'
-  // block (at most 128 rows x 16 streams) takes kSeqMaxRed elements per
-  // epilogue thread at most
+  // the fewest streams per cluster (16: one chain, 32: two chains of 16) whose
+  // clusters of 4 (or 2) CTAs fit in one wave, else 64 in one chain; each CTA
+  // owns 4, 8 or 16 streams of a chain, so its tau' block (at most 128 rows x
+  // 16 streams) takes kSeqMaxRed elements per epilogue thread at most
   const long long tiles16 = (B + 15) / 16, tiles32 = (B + 31) / 32;
   switch (H) {
     case 256: *ns = tiles16 <= 2 * kSeqMaxClusters4 ? 16 : 32; *mt = 1; return true;  // 2 CTAs x 128 units
