@@ -482,8 +482,9 @@ struct TcLoopArgs : TcLoopPlan {
   long long limit_ns;
   int test_stall;            // 1: CTA 0 withholds its first h (the waits run out)
 };
-// Whether a layer of this shape takes the resident-factor launch, and how.
-bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out);
+// Whether a layer of this shape takes the resident-factor launch, and how; slower_too: also some shapes that the
+// launches per step serve faster (for a run that may not allocate what those need).
+bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, bool slower_too, TcLoopPlan* out);
 // V: the V_h map whose boxes have a.vbox rows; U: U in boxes of 128 rows; Hm, Taum: h and tau' as planes
 // (tc_make_map_planes, boxes of p.nt rows).  *resident = false (and nothing launched) if the device
 // cannot hold the whole grid at once.

@@ -1109,7 +1109,7 @@ cudaError_t launch_loop_t(const TcMap& V, const TcMap& U, const TcMap& Hm, const
 
 }  // namespace
 
-bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
+bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, bool slower_too, TcLoopPlan* out) {
   if (H < 1 || H > 2048 || K < 1 || K > 1024 || B < 1 || B > kLoopMaxTiles * 16) return false;
   TcLoopPlan p{};
   p.rpg = K <= 16 ? 16 : K <= 32 ? 32 : K <= 64 ? 64 : 128;
@@ -1182,11 +1182,13 @@ bool tc_loop_plan(int H, int B, int K, const Checkpoints& ck, TcLoopPlan* out) {
   // - tiles of 16 in place of 32 for want of room: 128 with depths, else 64.  H = 2048, K = 1000, two depths, 96
   //   (B = 64) 306 / 364, 144 (B = 96) 429 / 406; H = 1024, K = 1000, no depths, 80 (B = 96) 240 / 235, 96 251 / 230.
   int limit = 192;
-  if (K > 512)
+  if (slower_too)
+    limit = 224;
+  else if (K > 512)
     limit = p.ga == 2 && K > 704 && p.ndep == 0 ? 128 : 160;
   else if (p.gp == 1 && p.ga <= 2 && p.ndep == 0 && K <= (p.ga == 2 ? 448 : 384))
     limit = 128;
-  const int limit16 = first == 16 ? limit : p.ndep > 0 ? 128 : 64;
+  const int limit16 = first == 16 || slower_too ? limit : p.ndep > 0 ? 128 : 64;
   // fills in the tile width nt with ures 64-term chunks of U in tensor memory; false if it does not fit
   auto fit = [&](int nt, int ures, TcLoopPlan* o) {
     TcLoopPlan c = p;

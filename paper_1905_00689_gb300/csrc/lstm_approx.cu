@@ -482,8 +482,15 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
   h->last_tensor_seq = 0;
   TcLoopPlan lp;
   const TensorTiles tt = tensor_tiles(H, B, K, ck);
-  if (h->opt_tensor_seq == 0 && h->opt_tau_layout == 0 && tc_loop_plan(H, B, K, ck, &lp) &&
-      loop_pays(lp, tt, H, B, K, T, ck)) {
+  // the launches per step may need raw sums' storage; a stream being captured cannot allocate it, the
+  // resident-factor launch needs none
+  const size_t raw_bytes = tt.raw ? (size_t)(tt.ks + ck.n) * 4 * B * H * sizeof(float) : 0;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (raw_bytes > h->gpart_bytes && cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess)
+    capture = cudaStreamCaptureStatusActive;
+  const bool no_storage = capture != cudaStreamCaptureStatusNone;
+  if (h->opt_tensor_seq == 0 && h->opt_tau_layout == 0 && tc_loop_plan(H, B, K, ck, no_storage, &lp) &&
+      (no_storage || loop_pays(lp, tt, H, B, K, T, ck))) {
     // one launch over all stream tiles for all T timesteps, the factors resident (offsets within a
     // timestep's P are 32-bit there: B * ldp below 2^31 follows from its limits on B and K)
     TcMap mh, mt;
@@ -544,17 +551,14 @@ int run_layer_tensor(lstm_approx_t* h, int l, const float* x, int T, int B, int 
   if (rpg > 0)
     LA_CUDA(h, cudaMemsetAsync(tau, 0, 2ull * B * 4 * h->Ks * sizeof(__nv_bfloat16), h->stream), "tau' clear");
   const int bnh = tt.bnh, nt = tt.nt, ks = tt.ks, nkb_per = tt.nkb_per;
-  if (tt.raw) {
-    const size_t need = (size_t)(ks + ck.n) * 4 * B * H * sizeof(float);
-    if (need > h->gpart_bytes) {
-      LA_CUDA(h, cudaStreamSynchronize(h->stream), "synchronising before growing the split buffer");
-      dfree(h, h->gpart, h->gpart_bytes);
-      h->gpart = nullptr;
-      h->gpart_bytes = 0;
-      rc = dmalloc(h, reinterpret_cast<void**>(&h->gpart), need, "split gate sums");
-      if (rc) return rc;
-      h->gpart_bytes = need;
-    }
+  if (raw_bytes > h->gpart_bytes) {
+    LA_CUDA(h, cudaStreamSynchronize(h->stream), "synchronising before growing the split buffer");
+    dfree(h, h->gpart, h->gpart_bytes);
+    h->gpart = nullptr;
+    h->gpart_bytes = 0;
+    rc = dmalloc(h, reinterpret_cast<void**>(&h->gpart), raw_bytes, "split gate sums");
+    if (rc) return rc;
+    h->gpart_bytes = raw_bytes;
   }
   TcMap mh, mt;
   if (!tc_make_map(&mh, hb, H, 2ull * B, (uint64_t)h->ldh * 2, bnh) ||
@@ -1440,7 +1444,7 @@ int lstm_approx_plan(int dtype, int hidden, int T, int B, int K, const int* chec
       v[LSTM_APPROX_PLAN_TAU_SPLITS] = tt.sk;
       TcLoopPlan lp;
       v[LSTM_APPROX_PLAN_TENSOR_LOOP] =
-          tc_loop_plan(hidden, B, K, ck, &lp) && loop_pays(lp, tt, hidden, B, K, T, ck) ? 1 : 0;
+          tc_loop_plan(hidden, B, K, ck, false, &lp) && loop_pays(lp, tt, hidden, B, K, T, ck) ? 1 : 0;
     }
   }
   for (int i = 0; i < n_out; ++i) out[i] = i < LSTM_APPROX_PLAN_ITEMS ? v[i] : 0;

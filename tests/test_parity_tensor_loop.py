@@ -94,6 +94,41 @@ def test_two_layers_and_graph_replay(cuda_device):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("H,B,K,T,warm", [
+    (256, 64, 1000, 2, (9, 1000)),    # few timesteps after many
+    (1024, 128, 1000, 9, (9, 512)),   # past this launch's limits after a shape within them
+])
+def test_capture_needs_no_storage_of_the_other_launches(cuda_device, H, B, K, T, warm):
+    """Where the launches per step are the faster way but would have to
+    allocate while the stream is captured, this launch is captured instead; an
+    eager run of the same call takes them."""
+    import torch
+    D = 40
+    gates = _gates(H, D + H, K, 60, 8900 + H)
+    x = torch.from_numpy(draw_inputs(warm[0], B, D, "uniform", 89).astype(np.float32)).cuda()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        m = LSTMApprox(1, [D], H, K, B, "bf16", stream=s)
+        m.set_layer(0, gates)
+        out = torch.empty(warm[0], B, H, device="cuda")
+        m.run(x, warm[1], out)
+        m.sync()
+        assert m.query(Q_TENSOR_LOOP) == 1
+        got = torch.empty(T, B, H, device="cuda")
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            m.run(x[:T], K, got)
+        assert m.query(Q_TENSOR_LOOP) == 1
+        g.replay()
+        m.sync()
+        eager = torch.empty(T, B, H, device="cuda")
+        m.run(x[:T], K, eager)
+        m.sync()
+        assert m.query(Q_TENSOR_LOOP) == 0 == plan(BF16, H, T, B, K, [])["tensor_loop"]
+    assert float((got - eager).abs().max()) <= 4e-4 * float(eager.abs().max())
+
+
+@pytest.mark.gpu
 def test_two_handles_on_two_streams(cuda_device):
     """Launches of two handles on two streams, each needing most of the SMs
     at once, complete and agree."""

@@ -41,10 +41,10 @@ int main() {
   const int Hs[] = {1, 63, 64, 65, 127, 128, 129, 301, 512, 513, 640, 1000, 1024, 1025, 1100, 1536, 2047, 2048};
   const int Ks[] = {1, 15, 16, 17, 32, 33, 64, 65, 90, 127, 128, 129, 200, 255, 256, 300, 512, 513, 640, 800, 902, 1000, 1023, 1024};
   const int Bs[] = {1, 2, 15, 16, 17, 31, 32, 33, 64, 65, 100, 128, 256, 300, 511, 700, 1024, 2000, 4096};
-  for (int H : Hs) for (int K : Ks) for (int B : Bs) for (int rep = 0; rep < 12; ++rep) {
+  for (int H : Hs) for (int K : Ks) for (int B : Bs) for (int rep = 0; rep < 12; ++rep) for (bool slower_too : {false, true}) {
     Checkpoints ck = rep == 0 ? Checkpoints{} : depths(K, &seed);
     TcLoopPlan p;
-    if (!tc_loop_plan(H, B, K, ck, &p)) continue;
+    if (!tc_loop_plan(H, B, K, ck, slower_too, &p)) continue;
     ++plans;
     const int gb = 4 / p.gp, nkb = (K + 63) / 64, nsl = (K + 15) / 16;
     CHECK(p.nt == 16 || p.nt == 32);
